@@ -28,7 +28,17 @@ DEVICE_SRC = ["kernels.cu", "noalloc.cu"]
 
 def _sources():
     return [os.path.join(CSRC, f) for f in HOST_SRC + DEVICE_SRC] + [
-        os.path.join(CSRC, "internal.h"), os.path.join(INCLUDE, "cusadi.h")]
+        os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "math64.cuh"),
+        os.path.join(INCLUDE, "cusadi.h")]
+
+
+def _embed_math() -> None:
+    """csrc/math64.cuh as a C++ string, compiled into the generated kernels that use it."""
+    with open(os.path.join(CSRC, "math64.cuh")) as f:
+        text = f.read()
+    lines = "".join('"' + ln.replace("\\", "\\\\").replace('"', '\\"') + '\\n"\n' for ln in text.split("\n"))
+    with open(os.path.join(OBJ, "math64_text.h"), "w") as f:
+        f.write("static const char* const kMath64Text =\n" + lines + ";\n")
 
 
 def _stale() -> bool:
@@ -45,7 +55,7 @@ def _compile(src: str) -> str:
                "-Xcompiler", "-fPIC", "-I", INCLUDE, "-c", src, "-o", obj]
     else:
         cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-Wall", "-I", INCLUDE,
-               "-I", os.path.join(CUDA, "include"), "-c", src, "-o", obj]
+               "-I", OBJ, "-I", os.path.join(CUDA, "include"), "-c", src, "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError(f"compile failed: {' '.join(cmd)}\n{r.stdout}\n{r.stderr}")
@@ -57,6 +67,7 @@ def build(force: bool = False) -> str:
     if not force and not _stale():
         return LIB
     os.makedirs(OBJ, exist_ok=True)
+    _embed_math()
     srcs = [os.path.join(CSRC, f) for f in DEVICE_SRC + HOST_SRC]
     with ThreadPoolExecutor(max_workers=len(srcs)) as ex:
         objs = list(ex.map(_compile, srcs))

@@ -27,6 +27,7 @@
 #include <sstream>
 
 #include "internal.h"
+#include "math64_text.h"   // kMath64Text: csrc/math64.cuh as text (made by the build)
 
 namespace cusadi {
 
@@ -74,6 +75,7 @@ MathFn math_name(int op) {
     case LOG1P: return {"log1p", "log1pf"};
     case EXPM1: return {"expm1", "expm1f"};
     case SQRT: return {"sqrt", "sqrtf"};
+    case DIV: case INV: return {"div", "div"};
     case FABS: return {"fabs", "fabsf"};
     case FMIN: return {"fmin", "fminf"};
     case FMAX: return {"fmax", "fmaxf"};
@@ -94,6 +96,7 @@ struct Gen {
   std::set<std::pair<int, bool>> calls;        // (op, f64) of out-of-line math used
   std::set<std::pair<int, bool>> calls2;       // (op, f64) of the paired (two-argument) versions
   bool own_f32 = false;                        // own FP32 sin/cos/exp used
+  bool own_f64 = false;                        // FP64 math of math64.cuh used
 
   Gen(const Graph& g_, const CodegenOptions& o_) : g(g_), o(o_) {}
 
@@ -116,6 +119,14 @@ bool inlined(int op, int inline_math) {
   return false;
 }
 
+// FP64 functions that run on the integer pipe (math64.cuh), where the
+// straight-line kernels leave it idle; an FP64 instruction occupies its unit 64
+// clocks per warp.  Weights in FMAs, library -> ours (see math64.cuh): exp 15,
+// sin/cos 18, div 7.7, sqrt 8.2 -> 1.6 to 4.
+bool own_f64_math(int op) {
+  return op == EXP || op == SIN || op == COS || op == DIV || op == INV || op == SQRT;
+}
+
 // __launch_bounds__ of a kernel of `threads` threads per CTA: a register cap
 // becomes the minimum number of resident CTAs per SM that leaves each thread
 // at most that many registers (a plain --maxrregcount is ignored for kernels
@@ -126,9 +137,32 @@ std::string launch_bounds(int threads, int maxrregcount) {
   return s + ")";
 }
 
+// Register cap of a one-thread kernel when the caller names none; 0 leaves it
+// to the compiler.  live: 32-bit registers' worth of values live at once; a
+// kernel needs about 20 more.
+//  * above the 255 a thread can have, the cap is 255: with calls to out-of-line
+//    functions the compiler else settles on as few as 32 registers and spills
+//    the rest (LQR step, 510 live: 179 KB of spill stores at 32 registers and
+//    1.24 ms, 33 KB at 255; MPC mixed 1.65 -> 1.35 ms);
+//  * 129 to 168 would hold 12 warps per SM, at most 128 holds 16: cap 128 (FP32
+//    random 20k-op program at N = 65,536, 165 registers: 0.61 -> 0.37 ms; FP64
+//    cart-pole, 138 registers: 0.075 -> 0.059 ms).
+int auto_register_cap(int64_t live) {
+  const int64_t need = live + 20;
+  if (need > 255) return 255;
+  return need > 128 && need <= 168 ? 128 : 0;
+}
+
+// the function itself, to be inlined where it is named
+std::string math_fn(int op, bool f64) {
+  MathFn m = math_name(op);
+  if (f64 && own_f64_math(op)) return std::string("cs_") + m.d + "64";
+  return f64 ? m.d : m.f;
+}
+
 std::string call_name(int op, bool f64, bool inl) {
   MathFn m = math_name(op);
-  if (inl) return f64 ? m.d : m.f;
+  if (inl) return math_fn(op, f64);
   return std::string("cs_") + m.d + (f64 ? "_d" : "_f");
 }
 
@@ -239,6 +273,13 @@ std::string op_expr(Gen& G, const Node& x, bool f, const std::string& A, const s
   std::string e;
   MathFn m = math_name(x.op);
   const char* mn = f ? m.d : m.f;
+  if (f && own_f64_math(x.op)) {
+    const int op = x.op == INV ? (int)DIV : (int)x.op;
+    const bool inl = inlined(op, o.inline_math);
+    if (!inl) G.calls.insert({op, true});
+    G.own_f64 = true;
+    return call_name(op, true, inl) + "(" + (x.op == INV ? One + ", " : "") + A + (x.op == DIV ? ", " + B : "") + ")";
+  }
   switch (x.op) {
     case ADD: e = A + " + " + B; break;
     case SUB: e = A + " - " + B; break;
@@ -430,6 +471,11 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   // the buffers allow it.  A kernel thread past the end of the batch still runs
   // (CTA barriers need it) on the last thread's instances, storing nothing.
   const int NL = o.device_fn ? 1 : std::max(1, o.inst_per_thread);
+  int cap = o.maxrregcount;
+  if (cap == 0 && !o.device_fn && !spill) {
+    int64_t words = o.dtype == CUSADI_F64 ? 2 : 1;   // MIXED: most values are single
+    cap = auto_register_cap(max_live(g) * words * NL);
+  }
   const bool clamped = o.adjoint || NL > 1 || (o.sync_every > 0 && !o.device_fn);
   R.inst_per_thread = NL;
   auto vname = [&](int64_t i, int r) {
@@ -478,6 +524,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     G.calls.clear();
     G.calls2.clear();
     G.own_f32 = false;
+    G.own_f64 = false;
     auto operand = [&](int32_t i, bool want_f64, int r) -> std::string {
       const Node& x = g.nodes[i];
       bool f = G.node_f64(i);
@@ -634,20 +681,20 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     src << "\n";
     if (NL > 1) src << kLaneAccess;
     if (G.own_f32) src << own_math_source(o.own_math);
+    if (G.own_f64) src << kMath64Text;
     if (o.debug_checks && !o.device_fn) src << "__device__ unsigned int cs_dbg;   // non-finite results\n";
     {
       for (auto& c : G.calls) {
-        MathFn m = math_name(c.first);
         const char* t = c.second ? "double" : "float";
         bool bin = op_arity(c.first) == 2;
         src << "static __device__ __noinline__ " << t << " " << call_name(c.first, c.second, false) << "("
             << t << " a" << (bin ? std::string(", ") + t + " b" : "") << ") { return "
-            << (c.second ? m.d : m.f) << "(a" << (bin ? ", b" : "") << "); }\n";
+            << math_fn(c.first, c.second) << "(a" << (bin ? ", b" : "") << "); }\n";
       }
       for (auto& c : G.calls2) {   // two independent evaluations per call
         MathFn m = math_name(c.first);
         const char* t = c.second ? "double" : "float";
-        const char* fn = c.second ? m.d : m.f;
+        const std::string fn = math_fn(c.first, c.second);
         src << "static __device__ __noinline__ " << t << "2 cs_" << m.d << "2" << (c.second ? "_d" : "_f")
             << "(" << t << " a, " << t << " b) { " << t << "2 r; r.x = " << fn << "(a); r.y = " << fn
             << "(b); return r; }\n";
@@ -676,7 +723,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       R.segs.push_back(std::move(S));
       continue;
     }
-    src << "extern \"C\" __global__ void " << launch_bounds(o.block, o.maxrregcount) << " " << name << "(\n"
+    src << "extern \"C\" __global__ void " << launch_bounds(o.block, cap) << " " << name << "(\n"
         << "    const " << tin << "* __restrict__ X, long long ldx, const " << tin
         << "* __restrict__ X2, long long ldx2, " << tin
         << "* __restrict__ Y, long long ldy,\n    long long N, " << tw
@@ -881,6 +928,7 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
     std::ostringstream regions;
     G.calls.clear();
     G.own_f32 = false;
+    G.own_f64 = false;
     const int nph_seg = segs[s].second - segs[s].first;
     // phase-major layout: every warp reaches the same __syncthreads() (aligned
     // barrier); a value used by its own warp in a later phase is declared once
@@ -986,15 +1034,15 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
     src << "// Generated cooperative kernel: segment " << s << " of " << nseg << ", " << W
         << " warps per 32 instances, " << (segs[s].second - segs[s].first) << " phases\n";
     if (G.own_f32) src << own_math_source(o.own_math);
+    if (G.own_f64) src << kMath64Text;
     if (o.debug_checks && !o.device_fn) src << "__device__ unsigned int cs_dbg;   // non-finite results\n";
     {
       for (auto& c : G.calls) {
-        MathFn m = math_name(c.first);
         const char* t = c.second ? "double" : "float";
         bool bin = op_arity(c.first) == 2;
         src << "static __device__ __noinline__ " << t << " " << call_name(c.first, c.second, false) << "("
             << t << " a" << (bin ? std::string(", ") + t + " b" : "") << ") { return "
-            << (c.second ? m.d : m.f) << "(a" << (bin ? ", b" : "") << "); }\n";
+            << math_fn(c.first, c.second) << "(a" << (bin ? ", b" : "") << "); }\n";
       }
     }
     std::string name = o.prefix + "_" + std::to_string(s);

@@ -16,6 +16,19 @@
 namespace cusadi {
 namespace {
 
+#include "math64.cuh"   // FP64 exp, sin, cos, division, square root on the integer pipe
+
+__device__ __forceinline__ double op_exp(double a) { return cs_exp64(a); }
+__device__ __forceinline__ double op_sin(double a) { return cs_sin64(a); }
+__device__ __forceinline__ double op_cos(double a) { return cs_cos64(a); }
+__device__ __forceinline__ double op_sqrt(double a) { return cs_sqrt64(a); }
+__device__ __forceinline__ double op_div(double a, double b) { return cs_div64(a, b); }
+__device__ __forceinline__ float op_exp(float a) { return expf(a); }
+__device__ __forceinline__ float op_sin(float a) { return sinf(a); }
+__device__ __forceinline__ float op_cos(float a) { return cosf(a); }
+__device__ __forceinline__ float op_sqrt(float a) { return sqrtf(a); }
+__device__ __forceinline__ float op_div(float a, float b) { return a / b; }
+
 constexpr int kInterpBlock = 128;   // threads per CTA of the interpreter kernel
 
 template <typename T>
@@ -25,15 +38,15 @@ __device__ __forceinline__ T eval_op(uint32_t op, T a, T b, T k) {
     case ADD: return a + b;
     case SUB: return a - b;
     case MUL: return a * b;
-    case DIV: return a / b;
+    case DIV: return op_div(a, b);
     case NEG: return -a;
-    case EXP: return exp(a);
+    case EXP: return op_exp(a);
     case LOG: return log(a);
     case POW: return pow(a, b);
     case SQ: return a * a;
-    case SQRT: return sqrt(a);
-    case SIN: return sin(a);
-    case COS: return cos(a);
+    case SQRT: return op_sqrt(a);
+    case SIN: return op_sin(a);
+    case COS: return op_cos(a);
     case TAN: return tan(a);
     case ATAN: return atan(a);
     case ATAN2: return atan2(a, b);
@@ -59,7 +72,7 @@ __device__ __forceinline__ T eval_op(uint32_t op, T a, T b, T k) {
     case FLOOR: return floor(a);
     case CEIL: return ceil(a);
     case FMOD: return fmod(a, b);
-    case INV: return O / a;
+    case INV: return op_div(O, a);
     case HYPOT: return hypot(a, b);
     case LOG1P: return log1p(a);
     case EXPM1: return expm1(a);
