@@ -407,7 +407,7 @@ cusadi_status cusadi_batch_create(const void* const* irs, const size_t* nbytes, 
         cc.device_fn = false;
         cc.prefix = "cs_bs" + std::to_string(p);
         cc.maxrregcount = o.maxrregcount;
-        P.scg = generate_coop(P.g, cc, plan_coop(P.g, o.ways, 8.0));
+        P.scg = generate_coop(P.g, cc, plan_coop(P.g, o.ways, 8.0, o.dtype));
       }
       P.ldw = (P.N + 31) / 32 * 32;
       b->ws_bytes = (b->ws_bytes + 255) / 256 * 256;

@@ -25,39 +25,48 @@ namespace cusadi {
 
 namespace {
 
-double op_cost(int op) {
-  switch (op) {
-    case SIN: case COS: case TAN: case ATAN: case ATAN2: case TANH: case ASIN: case ACOS:
+// Cost of one node in units of about 5 clocks (an FP32 add's latency).  FP64:
+// 64 clocks of the FP64 unit per add or multiply, the measured latency of the
+// integer-pipe functions (math64.cuh: division 344, square root 298, exp 408,
+// sin/cos 551 clocks), the library's for the rest.
+double op_cost(const Node& x, int dtype) {
+  const bool f64 = dtype == CUSADI_F64 || (dtype == CUSADI_MIXED && x.f64);
+  switch (x.op) {
+    case SIN: case COS:
+      return f64 ? 110.0 : 24.0;
+    case TAN: case ATAN: case ATAN2: case TANH: case ASIN: case ACOS:
     case SINH: case COSH: case ERF: case POW: case LOG: case HYPOT: case LOG1P: case EXPM1:
     case FMOD:
-      return 24.0;
-    case EXP: return 12.0;
-    case DIV: case SQRT: case INV: return 8.0;
-    default: return 1.0;
+      return f64 ? 300.0 : 24.0;
+    case EXP: return f64 ? 80.0 : 12.0;
+    case DIV: case SQRT: case INV: return f64 ? 65.0 : 8.0;
+    default: return f64 ? 13.0 : 1.0;
   }
 }
 
 // a CTA barrier plus the shared-memory hand-off, in op costs (CUSADI_COOP_BARRIER_COST
-// overrides it, for sweeps of the phase count against compile time and run time)
-double barrier_cost() {
+// overrides it, for sweeps of the phase count against compile time and run time);
+// FP64: six adds, as for FP32 (random 20k program, N = 4,096, 8 warps: 272 us from
+// 20 to 150 units here, 317 us at 6)
+double barrier_cost(int dtype) {
   static const double c = [] {
     const char* e = std::getenv("CUSADI_COOP_BARRIER_COST");
-    return e ? std::max(0.0, std::atof(e)) : 6.0;
+    return e ? std::max(0.0, std::atof(e)) : -1.0;
   }();
-  return c;
+  return c >= 0 ? c : (dtype == CUSADI_F64 ? 78.0 : 6.0);
 }
 
 bool is_leaf(const Graph& g, int64_t i) { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; }
 
 // sum over phases of (the busiest warp's op cost + one barrier)
-double estimate(const Graph& g, const CoopPlan& P) {
+double estimate(const Graph& g, const CoopPlan& P, const std::vector<double>& cost, int dtype) {
   std::vector<double> load((size_t)P.n_phases * P.ways, 0.0);
   for (int64_t i = 0; i < (int64_t)g.nodes.size(); ++i)
-    if (!is_leaf(g, i)) load[(size_t)P.phase[i] * P.ways + P.owner[i]] += op_cost(g.nodes[i].op);
+    if (!is_leaf(g, i)) load[(size_t)P.phase[i] * P.ways + P.owner[i]] += cost[i];
   double t = 0;
   for (int q = 0; q < P.n_phases; ++q)
     t += *std::max_element(load.begin() + (size_t)q * P.ways, load.begin() + (size_t)(q + 1) * P.ways) +
-         barrier_cost();
+         barrier_cost(dtype);
   return t;
 }
 
@@ -67,7 +76,8 @@ struct Ready {
   bool operator<(const Ready& o) const { return pri < o.pri || (pri == o.pri && i > o.i); }
 };
 
-CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<double>& bottom,
+CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<double>& cost,
+                     const std::vector<double>& bottom,
                      const std::vector<std::vector<int64_t>>& users) {
   const int64_t n = (int64_t)g.nodes.size();
   CoopPlan P;
@@ -101,7 +111,7 @@ CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<
       if (!has_mine && !has_open) { full[w] = 1; --active; continue; }
       const bool take_mine = has_mine && (!has_open || !(mine[w].top() < open.top()));
       const Ready r = take_mine ? mine[w].top() : open.top();
-      const double c = op_cost(g.nodes[r.i].op);
+      const double c = cost[r.i];
       if (load[w] > 0 && load[w] + c > target) { full[w] = 1; --active; continue; }
       (take_mine ? mine[w] : open).pop();
       P.owner[r.i] = w;
@@ -130,31 +140,36 @@ CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<
   return P;
 }
 
-CoopPlan plan_eft(const Graph& g, int ways, double comm_cost);
+CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost);
 
 }  // namespace
 
-CoopPlan plan_coop(const Graph& g, int ways, double comm_cost) {
+CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
   const int64_t n = (int64_t)g.nodes.size();
+  std::vector<double> cost(n, 0.0);
+  for (int64_t i = 0; i < n; ++i)
+    if (!is_leaf(g, i)) cost[i] = op_cost(g.nodes[i], dtype);
   // bottom level: op cost on the longest path from the op to the end
   std::vector<double> bottom(n, 0.0);
   std::vector<std::vector<int64_t>> users(n);
   for (int64_t i = 0; i < n; ++i) {
     if (is_leaf(g, i)) continue;
-    bottom[i] = op_cost(g.nodes[i].op);
+    bottom[i] = cost[i];
     for (int32_t o : {g.nodes[i].a, g.nodes[i].b})
       if (o >= 0 && !is_leaf(g, o)) users[o].push_back(i);
   }
   for (int64_t i = n - 1; i >= 0; --i) {
     if (is_leaf(g, i)) continue;
     for (int32_t o : {g.nodes[i].a, g.nodes[i].b})
-      if (o >= 0 && !is_leaf(g, o)) bottom[o] = std::max(bottom[o], op_cost(g.nodes[o].op) + bottom[i]);
+      if (o >= 0 && !is_leaf(g, o)) bottom[o] = std::max(bottom[o], cost[o] + bottom[i]);
   }
-  CoopPlan best = plan_eft(g, ways, comm_cost);
-  double best_t = estimate(g, best);
+  CoopPlan best = plan_eft(g, ways, comm_cost, cost);
+  double best_t = estimate(g, best, cost, dtype);
+  // FP64 phases hold as many ops at 13 times the cost
+  const double unit = dtype == CUSADI_F64 ? 13.0 : 1.0;
   for (double target : {8.0, 16.0, 32.0, 64.0, 128.0, 256.0, 512.0}) {
-    CoopPlan P = plan_packed(g, ways, target, bottom, users);
-    const double t = estimate(g, P);
+    CoopPlan P = plan_packed(g, ways, target * unit, cost, bottom, users);
+    const double t = estimate(g, P, cost, dtype);
     if (t < best_t) { best_t = t; best = std::move(P); }
   }
   return best;
@@ -162,7 +177,7 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost) {
 
 namespace {
 
-CoopPlan plan_eft(const Graph& g, int ways, double comm_cost) {
+CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost) {
   const int64_t n = (int64_t)g.nodes.size();
   CoopPlan P;
   P.ways = ways;
@@ -179,7 +194,7 @@ CoopPlan plan_eft(const Graph& g, int ways, double comm_cost) {
       double start = avail[w];
       for (int32_t o : {x.a, x.b})
         if (o >= 0 && !leaf(o)) start = std::max(start, finish[o] + (P.owner[o] == w ? 0.0 : comm_cost));
-      double f = start + op_cost(x.op);
+      double f = start + cost[i];
       if (f < best_f - 1e-12 || (f < best_f + 1e-12 && avail[w] < avail[best])) {
         best = w;
         best_f = f;

@@ -139,7 +139,7 @@ struct CoopPlan {
   std::vector<int> phase;        // per node: barrier-separated phase
   int n_phases = 1;
 };
-CoopPlan plan_coop(const Graph& g, int ways, double comm_cost);
+CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype);
 // Shared-memory slots (at most max_slots; overflow to workspace rows gslot) of
 // the values read by another warp of the same kernel (seg_of_node: kernel of
 // each node); returns the shared slot count.

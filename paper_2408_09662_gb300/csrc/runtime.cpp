@@ -233,7 +233,7 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   if (fn->opt.ways > 1) {
     co.prefix = std::string(adjoint ? "cs_coopadj" : "cs_coop") + std::to_string(fn->opt.ways) + "_" +
                 tag[fn->opt.dtype];
-    CoopPlan plan = plan_coop(d.g, fn->opt.ways, 8.0);
+    CoopPlan plan = plan_coop(d.g, fn->opt.ways, 8.0, fn->opt.dtype);
     // the CTA's groups share the shared-memory budget
     co.coop_shared_kb = std::min(co.coop_shared_kb, 200 / std::max(1, co.coop_groups));
     d.cg = generate_coop(d.g, co, plan);
