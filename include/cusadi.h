@@ -63,9 +63,10 @@ typedef enum { CUSADI_F64 = 0, CUSADI_F32 = 1, CUSADI_MIXED = 2 } cusadi_dtype;
 
 /* Evaluation path.  COMPILED: generated straight-line CUDA kernels (one
  * instance per thread, values in registers).  INTERP: one precompiled kernel
- * that walks a packed instruction stream (no compile time; for programs too
- * large to compile).  AUTO picks COMPILED up to compile_limit_ops, and the
- * interpreter when the program is larger or NVRTC fails on it. */
+ * whose warps walk packed instruction streams, several warps per group of 32
+ * instances (no compile time; for programs too large to compile).  AUTO picks
+ * COMPILED up to compile_limit_ops, and the interpreter when the program is
+ * larger or NVRTC fails on it. */
 typedef enum { CUSADI_PATH_AUTO = 0, CUSADI_PATH_COMPILED = 1, CUSADI_PATH_INTERP = 2 } cusadi_path;
 
 typedef struct {
@@ -111,12 +112,13 @@ typedef struct {
                                  after every this many ops, so the CTA's warps stay in
                                  the same stretch of a long kernel's code (instruction
                                  cache reuse); 0: no barriers                       (0) */
-  int32_t interp_shared_kb;   /* interpreter path: shared memory per 128-thread CTA for the
-                                 work slots, in KB (0..200); the slots of the values that
-                                 do not fit, chosen by linear scan as the ones read
-                                 last, live in the workspace; more shared memory
-                                 means fewer resident CTAs, which costs more than the
-                                 slots gain beyond ~48 KB on GB300                 (48) */
+  int32_t interp_shared_kb;   /* interpreter path: shared memory per 128 threads of a CTA
+                                 for the work slots, in KB (0..200; at most 200 per CTA);
+                                 the slots of the values that do not fit, chosen by
+                                 linear scan as the ones read last, live in the
+                                 workspace; more shared memory means fewer resident
+                                 CTAs, which costs more than the slots gain beyond
+                                 ~48 KB on GB300                                   (48) */
   int32_t spill_values;       /* one-thread-per-instance kernels (ways = 0, inst_per_thread
                                  = 1): > 0 keeps at most this many values live in
                                  registers; linear scan over their live ranges moves the

@@ -23,8 +23,6 @@
 
 namespace cusadi {
 
-namespace {
-
 // Cost of one node in units of about 5 clocks (an FP32 add's latency).  FP64:
 // 64 clocks of the FP64 unit per add or multiply, the measured latency of the
 // integer-pipe functions (math64.cuh: division 344, square root 298, exp 408,
@@ -44,6 +42,8 @@ double op_cost(const Node& x, int dtype) {
   }
 }
 
+namespace {
+
 // a CTA barrier plus the shared-memory hand-off, in op costs (CUSADI_COOP_BARRIER_COST
 // overrides it, for sweeps of the phase count against compile time and run time);
 // FP64: six adds, as for FP32 (random 20k program, N = 4,096, 8 warps: 272 us from
@@ -58,28 +58,44 @@ double barrier_cost(int dtype) {
 
 bool is_leaf(const Graph& g, int64_t i) { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; }
 
-// sum over phases of (the busiest warp's op cost + one barrier)
-double estimate(const Graph& g, const CoopPlan& P, const std::vector<double>& cost, int dtype) {
-  std::vector<double> load((size_t)P.n_phases * P.ways, 0.0);
-  for (int64_t i = 0; i < (int64_t)g.nodes.size(); ++i)
-    if (!is_leaf(g, i)) load[(size_t)P.phase[i] * P.ways + P.owner[i]] += cost[i];
-  double t = 0;
-  for (int q = 0; q < P.n_phases; ++q)
-    t += *std::max_element(load.begin() + (size_t)q * P.ways, load.begin() + (size_t)(q + 1) * P.ways) +
-         barrier_cost(dtype);
-  return t;
-}
-
 struct Ready {
   double pri;
   int64_t i;
   bool operator<(const Ready& o) const { return pri < o.pri || (pri == o.pri && i > o.i); }
 };
 
-CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<double>& cost,
-                     const std::vector<double>& bottom,
-                     const std::vector<std::vector<int64_t>>& users) {
-  const int64_t n = (int64_t)g.nodes.size();
+CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost);
+
+}  // namespace
+
+void PhaseDag::finish() {
+  const int64_t n = (int64_t)deps.size();
+  bottom.assign(n, 0.0);
+  users.assign(n, {});
+  for (int64_t i = 0; i < n; ++i) {
+    if (skip[i]) continue;
+    bottom[i] = cost[i];
+    for (int32_t o : deps[i])
+      if (o >= 0) users[o].push_back(i);
+  }
+  for (int64_t i = n - 1; i >= 0; --i)
+    if (!skip[i])
+      for (int32_t o : deps[i])
+        if (o >= 0) bottom[o] = std::max(bottom[o], cost[o] + bottom[i]);
+}
+
+double estimate_phases(const PhaseDag& d, const CoopPlan& P, double barrier) {
+  std::vector<double> load((size_t)P.n_phases * P.ways, 0.0);
+  for (int64_t i = 0; i < (int64_t)d.deps.size(); ++i)
+    if (!d.skip[i]) load[(size_t)P.phase[i] * P.ways + P.owner[i]] += d.cost[i];
+  double t = 0;
+  for (int q = 0; q < P.n_phases; ++q)
+    t += *std::max_element(load.begin() + (size_t)q * P.ways, load.begin() + (size_t)(q + 1) * P.ways) + barrier;
+  return t;
+}
+
+CoopPlan pack_phases(const PhaseDag& d, int ways, double target) {
+  const int64_t n = (int64_t)d.deps.size();
   CoopPlan P;
   P.ways = ways;
   P.owner.assign(n, -1);
@@ -90,11 +106,11 @@ CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<
   std::vector<std::priority_queue<Ready>> mine(ways);     // need a value of this warp's phase
   std::vector<int64_t> later;                             // need values of two warps' phase
   for (int64_t i = 0; i < n; ++i) {
-    if (is_leaf(g, i)) continue;
+    if (d.skip[i]) continue;
     ++todo;
-    for (int32_t o : {g.nodes[i].a, g.nodes[i].b})
-      if (o >= 0 && !is_leaf(g, o)) ++pending[i];
-    if (pending[i] == 0) open.push({bottom[i], i});
+    for (int32_t o : d.deps[i])
+      if (o >= 0) ++pending[i];
+    if (pending[i] == 0) open.push({d.bottom[i], i});
   }
   int q = 0;
   std::vector<double> load(ways);
@@ -111,28 +127,28 @@ CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<
       if (!has_mine && !has_open) { full[w] = 1; --active; continue; }
       const bool take_mine = has_mine && (!has_open || !(mine[w].top() < open.top()));
       const Ready r = take_mine ? mine[w].top() : open.top();
-      const double c = cost[r.i];
+      const double c = d.cost[r.i];
       if (load[w] > 0 && load[w] + c > target) { full[w] = 1; --active; continue; }
       (take_mine ? mine[w] : open).pop();
       P.owner[r.i] = w;
       P.phase[r.i] = q;
       load[w] += c;
       --todo;
-      for (int64_t u : users[r.i]) {
+      for (int64_t u : d.users[r.i]) {
         if (--pending[u] != 0) continue;
         int same = -1;   // warp of the operands computed in this phase, -2 if two warps
-        for (int32_t o : {g.nodes[u].a, g.nodes[u].b})
-          if (o >= 0 && !is_leaf(g, o) && P.phase[o] == q)
+        for (int32_t o : d.deps[u])
+          if (o >= 0 && P.phase[o] == q)
             same = (same == -1 || same == P.owner[o]) ? P.owner[o] : -2;
-        if (same == -1) open.push({bottom[u], u});
-        else if (same >= 0) mine[same].push({bottom[u], u});
+        if (same == -1) open.push({d.bottom[u], u});
+        else if (same >= 0) mine[same].push({d.bottom[u], u});
         else later.push_back(u);
       }
     }
     // what waited on this phase's values of one warp, or of two, is open next phase
     for (auto& m : mine)
       while (!m.empty()) { open.push(m.top()); m.pop(); }
-    for (int64_t u : later) open.push({bottom[u], u});
+    for (int64_t u : later) open.push({d.bottom[u], u});
     later.clear();
     ++q;
   }
@@ -140,36 +156,27 @@ CoopPlan plan_packed(const Graph& g, int ways, double target, const std::vector<
   return P;
 }
 
-CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost);
-
-}  // namespace
-
 CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
   const int64_t n = (int64_t)g.nodes.size();
-  std::vector<double> cost(n, 0.0);
-  for (int64_t i = 0; i < n; ++i)
-    if (!is_leaf(g, i)) cost[i] = op_cost(g.nodes[i], dtype);
-  // bottom level: op cost on the longest path from the op to the end
-  std::vector<double> bottom(n, 0.0);
-  std::vector<std::vector<int64_t>> users(n);
+  PhaseDag d;
+  d.deps.assign(n, {-1, -1, -1});
+  d.skip.assign(n, 0);
+  d.cost.assign(n, 0.0);
   for (int64_t i = 0; i < n; ++i) {
-    if (is_leaf(g, i)) continue;
-    bottom[i] = cost[i];
-    for (int32_t o : {g.nodes[i].a, g.nodes[i].b})
-      if (o >= 0 && !is_leaf(g, o)) users[o].push_back(i);
+    if (is_leaf(g, i)) { d.skip[i] = 1; continue; }
+    const Node& x = g.nodes[i];
+    d.cost[i] = op_cost(x, dtype);
+    if (x.a >= 0 && !is_leaf(g, x.a)) d.deps[i][0] = x.a;
+    if (x.b >= 0 && !is_leaf(g, x.b)) d.deps[i][1] = x.b;
   }
-  for (int64_t i = n - 1; i >= 0; --i) {
-    if (is_leaf(g, i)) continue;
-    for (int32_t o : {g.nodes[i].a, g.nodes[i].b})
-      if (o >= 0 && !is_leaf(g, o)) bottom[o] = std::max(bottom[o], cost[o] + bottom[i]);
-  }
-  CoopPlan best = plan_eft(g, ways, comm_cost, cost);
-  double best_t = estimate(g, best, cost, dtype);
+  d.finish();
+  CoopPlan best = plan_eft(g, ways, comm_cost, d.cost);
+  double best_t = estimate_phases(d, best, barrier_cost(dtype));
   // FP64 phases hold as many ops at 13 times the cost
   const double unit = dtype == CUSADI_F64 ? 13.0 : 1.0;
   for (double target : {8.0, 16.0, 32.0, 64.0, 128.0, 256.0, 512.0}) {
-    CoopPlan P = plan_packed(g, ways, target * unit, cost, bottom, users);
-    const double t = estimate(g, P, cost, dtype);
+    CoopPlan P = pack_phases(d, ways, target * unit);
+    const double t = estimate_phases(d, P, barrier_cost(dtype));
     if (t < best_t) { best_t = t; best = std::move(P); }
   }
   return best;

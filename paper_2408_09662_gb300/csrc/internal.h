@@ -1,6 +1,7 @@
 // Internal declarations of libcusadi: IR, SSA graph, passes, code generation.
 #pragma once
 
+#include <array>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -139,6 +140,21 @@ struct CoopPlan {
   std::vector<int> phase;        // per node: barrier-separated phase
   int n_phases = 1;
 };
+// Ops with their dependences and costs, for the phase-packing scheduler.
+struct PhaseDag {
+  std::vector<std::array<int32_t, 3>> deps;   // per op: ops whose results it reads (-1: none)
+  std::vector<uint8_t> skip;                  // not an op of its own (leaves, ops fused into another)
+  std::vector<double> cost;
+  // filled by finish(): critical path to the end, readers
+  std::vector<double> bottom;
+  std::vector<std::vector<int64_t>> users;
+  void finish();
+};
+// Fills one phase after the other, up to `target` cost per warp, with the ready
+// op of the longest remaining critical path.
+CoopPlan pack_phases(const PhaseDag& d, int ways, double target);
+// Sum over phases of the busiest warp's cost plus a barrier.
+double estimate_phases(const PhaseDag& d, const CoopPlan& P, double barrier);
 CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype);
 // Shared-memory slots (at most max_slots; overflow to workspace rows gslot) of
 // the values read by another warp of the same kernel (seg_of_node: kernel of
@@ -150,17 +166,33 @@ int assign_coop_slots(const Graph& g, const CoopPlan& P, const std::vector<int>&
 CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopPlan& plan);
 
 // --- interpreter stream -------------------------------------------------------
-// code = op | f64 << 7 | bcast << 6 ... packed per instruction (see kernels.cu)
+// Cost of one op in units of about 5 clocks (coop.cpp).
+double op_cost(const Node& x, int dtype);
+
+// Instruction of the interpreter kernel (see kernels.cu).  code: bits 0..6 op,
+// bit 7 f64 tag, bits 8..31 destination slot (I_OUTPUT: output row).  a, b, c:
+// operands, bits 30..31 class (0 work slot, 1 input row, 2 broadcast input row,
+// 3 constant), bits 0..29 index; b of I_OUTPUT: index among the reduced rows + 1.
 struct IOp {
-  uint32_t code;   // bits 0..6 op, bit 7 f64 tag, bits 8..31 aux (input row / const / output row)
-  uint32_t out;    // destination slot (OUTPUT: unused)
-  uint32_t a, b;   // operand slots
+  uint32_t code, a, b, c;
 };
+// ops of the stream beside the program's: padding, a barrier between phases, an
+// output store, and a multiply (rounded) whose only reader is an add or subtract
+enum InterpOp : uint32_t { I_NOP = 64, I_SYNC, I_OUTPUT, I_MUL_ADD, I_MUL_SUB, I_SUB_MUL,
+                           // the same multiply-adds, in bundles made of nothing else (all work
+                           // slots in shared memory; any work slots)
+                           I_FAST = 96, I_FAST_FAR = 112 };
+// The stream is a sequence of bundles of this many instructions that do not read
+// one another's results.
+constexpr int kBundle = 4;
+constexpr uint32_t kOperandShift = 30, kOperandMask = (1u << kOperandShift) - 1;
 
 struct InterpProgram {
-  std::vector<IOp> ops;
+  std::vector<IOp> ops;            // the warps' streams, one after the other
   std::vector<double> k;
-  std::vector<uint8_t> in_bcast;
+  int ways = 1;                    // warps per group of 32 instances
+  double estimate = 0;             // cost of the layout (interp.cpp)
+  std::vector<int32_t> begin;      // ways + 1: first instruction of each warp's stream
   int64_t n_slots = 0;             // n_shared + n_global (at least 1)
   int64_t n_shared = 0;            // slots 0 .. n_shared - 1: shared memory
   int64_t n_global = 0;            // slots n_shared ..: rows of the global workspace
@@ -168,14 +200,16 @@ struct InterpProgram {
   std::vector<int64_t> reduce_rows;   // output rows summed over instances (adjoint)
 };
 
-// At most max_shared slots go to shared memory (interp.cpp: linear scan).
-bool pack_interp(const Graph& g, InterpProgram& p, std::string& err, int64_t max_shared);
-// Shared-memory slots per thread of the interpreter kernel for a budget in KB.
-int interp_shared_slots(int dtype, int shared_kb);
+// Schedules the program over warps and phases and places its values
+// (interp.cpp).  shared_kb: shared memory per 128 threads of a CTA for slots.
+bool pack_interp(const Graph& g, InterpProgram& many, InterpProgram& few, std::string& err, int dtype,
+                 int shared_kb);
+// Instances up to which `few` runs: a group of 32 per SM.
+constexpr int64_t kInterpFew = 152 * 32;
 
 // launchers implemented in kernels.cu.  Input rows >= split are read from X2
 // (row - split); returns a cudaError_t value.
-int launch_interp(const IOp* ops, int64_t n_ops, const double* k, int dtype, const void* X,
+int launch_interp(const IOp* ops, const int32_t* begin, int ways, const void* k, int dtype, const void* X,
                   int64_t ldx, const void* X2, int64_t ldx2, int64_t split, void* Y, int64_t ldy,
                   int64_t N, void* W, int64_t ldw, int64_t n_shared, int acc, int reduce,
                   void* Wr, int64_t ldr, void* stream);

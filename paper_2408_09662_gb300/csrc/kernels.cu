@@ -1,9 +1,10 @@
-// Interpreter kernel: one thread per instance walks a packed instruction
-// stream (the sequential traversal of CusADi §III-A), for programs that are too
-// large to compile.  Every thread reads the same instruction at the same time,
-// so the switch below never diverges within a warp.  The work vector lives in
-// shared memory (slot-major, one column per thread: conflict-free) when it
-// fits, else in a global workspace in the instance-fastest layout.
+// Interpreter kernel, for programs that are too large to compile: W warps walk
+// the instruction streams of one group of 32 instances (lane = instance), with
+// CTA barriers between the phases that the host laid out (interp.cpp).  Every
+// lane of a warp reads the same instruction, so the switch below never diverges
+// within a warp.  The work vector lives in shared memory (slot-major, one column
+// per lane: conflict-free) and, beyond that, in a global workspace in the
+// instance-fastest layout, of which one group's columns stay in L2.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -28,8 +29,6 @@ __device__ __forceinline__ float op_sin(float a) { return sinf(a); }
 __device__ __forceinline__ float op_cos(float a) { return cosf(a); }
 __device__ __forceinline__ float op_sqrt(float a) { return sqrtf(a); }
 __device__ __forceinline__ float op_div(float a, float b) { return a / b; }
-
-constexpr int kInterpBlock = 128;   // threads per CTA of the interpreter kernel
 
 template <typename T>
 __device__ __forceinline__ T eval_op(uint32_t op, T a, T b, T k) {
@@ -82,77 +81,162 @@ __device__ __forceinline__ T eval_op(uint32_t op, T a, T b, T k) {
   return Z;
 }
 
+__device__ __forceinline__ double flip(double v, uint32_t sign) {
+  return __hiloint2double((int)((uint32_t)__double2hiint(v) ^ sign), __double2loint(v));
+}
+__device__ __forceinline__ float flip(float v, uint32_t sign) {
+  return __uint_as_float(__float_as_uint(v) ^ sign);
+}
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+
+// a * b rounded on its own, then added to or subtracted from c (or c from it);
+// a subtraction is the addition of the negated operand, so the FP64 unit sees two
+// instructions whichever it is
+template <typename T>
+__device__ __forceinline__ T mul_then(uint32_t op, T a, T b, T c) {
+  return add_rn(flip(mul_rn(a, b), op == I_SUB_MUL ? 0x80000000u : 0u), flip(c, op == I_MUL_SUB ? 0x80000000u : 0u));
+}
+template <typename T>
+__device__ __forceinline__ T interp_op(uint32_t op, T a, T b, T c) {
+  if (op >= I_MUL_ADD) return mul_then(op, a, b, c);
+  return eval_op<T>(op, a, b, c);
+}
+
 // B: buffer element type; S: work-slot type; MIXED: per-op precision tags.
-// Slots below n_shared live in shared memory (slot-major, one column per
-// thread: conflict-free), the others in the global workspace (row s - n_shared,
-// instance-fastest); every slot index in the stream is warp-uniform, so the
-// tier test never diverges.
+// A warp stages its stream 32 instructions at a time: one coalesced load per lane,
+// issued a batch ahead, then broadcast reads.  Bundles of multiply-adds on work
+// slots, most of what linear algebra is made of, have their operands read together
+// and are evaluated without decoding; other instructions (about 100 issued each)
+// run one after the other.  Measured (GB300, ms; one thread per instance with the
+// slots in HBM -> this): LDL^T FP64 n = 47, N = 16,384 16.7 -> 2.81, n = 100, N =
+// 8,192 180 -> 15.5, n = 22, N = 65,536 2.36 -> 1.48; random 20k ops FP64, N =
+// 16,384 8.6 -> 2.2; MPC mixed 19.8 -> 5.1.  The FP64 unit's share is 1.3 ms of the
+// 2.81; barriers between phases and reads of workspace rows make up the rest.
+// (Programs of a few dozen ops lose: quadrotor Jacobian FP32, N = 1,000,003, 0.140
+// -> 0.155.)
 template <typename B, typename S, bool MIXED>
-__global__ void __launch_bounds__(kInterpBlock) interp_kernel(
-    const uint4* __restrict__ ops, long long n_ops, const double* __restrict__ K,
+__global__ void __launch_bounds__(512, 1) interp_kernel(
+    const uint4* __restrict__ ops, const int32_t* __restrict__ begin, int ways, const S* __restrict__ K,
     const B* __restrict__ X, long long ldx, const B* __restrict__ X2, long long ldx2,
-    long long split, B* __restrict__ Y, long long ldy, long long N, S* __restrict__ W,
+    long long split, B* __restrict__ Y, long long ldy, long long N, S* W,
     long long ldw, unsigned n_shared, int acc, int reduce, S* __restrict__ Wr, long long ldr) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const long long i0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  // one-warp groups come several to a CTA (their streams have no barriers)
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, warp = w % ways, grp = w / ways;
+  const long long i0 = ((long long)blockIdx.x * ((blockDim.x >> 5) / ways) + grp) * 32 + lane;
   const bool active = i0 < N;
   const long long ix = active ? i0 : N - 1;  // inactive lanes read a valid column
-  S* const sm = reinterpret_cast<S*>(smem_raw) + threadIdx.x;
-  S* const gm = W + i0;                      // columns up to the grid's end exist (ldw)
-  auto at = [&](unsigned s) -> S& {
-    return s < n_shared ? sm[(size_t)s * kInterpBlock] : gm[(long long)(s - n_shared) * ldw];
+  uint4* const stage = reinterpret_cast<uint4*>(smem_raw) + w * 64;
+  S* const sm = reinterpret_cast<S*>(reinterpret_cast<uint4*>(smem_raw) + (blockDim.x >> 5) * 64) +
+                grp * n_shared * 32 + lane;
+  S* const gm = W + i0;                      // columns up to the next multiple of 128 exist (ldw)
+  auto get = [&](unsigned o) -> S {
+    if (o < n_shared) return sm[o * 32];
+    const unsigned cls = o >> kOperandShift;
+    const long long k = o & kOperandMask;
+    if (cls == 0) return gm[(k - n_shared) * ldw];
+    if (cls == 3) return K[k];
+    const long long col = cls == 2 ? 0 : ix;
+    return (S)(k < split ? X[k * ldx + col] : X2[(k - split) * ldx2 + col]);
   };
-  for (long long t = 0; t < n_ops; ++t) {
-    const uint4 o = __ldg(&ops[t]);
-    const uint32_t op = o.x & 127u;
-    const long long aux = (long long)(o.x >> 8);
-    if (op == INPUT) {
-      const long long col = o.w ? 0 : ix;
-      at(o.y) = aux < split ? (S)X[aux * ldx + col] : (S)X2[(aux - split) * ldx2 + col];
-      continue;
-    }
-    if (op == CONST) {
-      at(o.y) = (S)K[aux];
-      continue;
-    }
-    if (op == OUTPUT) {
-      const S v = at(o.z);
-      if (o.w && reduce) {   // reduced row o.w - 1: the instance's term, summed later
-        if (active) Wr[(long long)(o.w - 1) * ldr + i0] = v;
-      } else if (active) {
-        B* p = &Y[aux * ldy + i0];
-        *p = acc ? *p + (B)v : (B)v;
+  auto any = [&](unsigned o) -> S* {         // a work slot of either tier
+    return o < n_shared ? sm + o * 32 : gm + (long long)(o - n_shared) * ldw;
+  };
+  const int end = begin[warp + 1];
+  int at = begin[warp];
+  uint4 next = at + lane < end ? ops[at + lane] : make_uint4(I_NOP, 0, 0, 0);
+  for (int turn = 0; at < end; at += 32, turn ^= 32) {
+    stage[turn + lane] = next;
+    __syncwarp();
+    next = at + 32 + lane < end ? ops[at + 32 + lane] : make_uint4(I_NOP, 0, 0, 0);
+    const int m = end - at < 32 ? end - at : 32;
+    uint4 ahead = stage[turn];
+    for (int t = 0; t < m;) {
+      const uint4 o = ahead;
+      const unsigned op = o.x & 127u, dst = o.x >> 8;
+      if (!MIXED && op >= I_FAST) {          // kBundle multiply-adds on work slots
+        const uint4* const d = stage + turn + t;
+        t += kBundle;
+        ahead = stage[turn + (t & 31)];
+        S a[kBundle], b[kBundle], c[kBundle];
+        unsigned code[kBundle];
+        if (op < I_FAST_FAR) {
+#pragma unroll
+          for (int j = 0; j < kBundle; ++j) {
+            const uint4 e = d[j];
+            code[j] = e.x;
+            a[j] = sm[e.y * 32];
+            b[j] = sm[e.z * 32];
+            c[j] = sm[e.w * 32];
+          }
+#pragma unroll
+          for (int j = 0; j < kBundle; ++j)
+            sm[(code[j] >> 8) * 32] = mul_then(I_MUL_ADD + (code[j] & 3u), a[j], b[j], c[j]);
+        } else {
+#pragma unroll
+          for (int j = 0; j < kBundle; ++j) {
+            const uint4 e = d[j];
+            code[j] = e.x;
+            a[j] = *any(e.y);
+            b[j] = *any(e.z);
+            c[j] = *any(e.w);
+          }
+#pragma unroll
+          for (int j = 0; j < kBundle; ++j)
+            *any(code[j] >> 8) = mul_then(I_MUL_ADD + (code[j] & 3u), a[j], b[j], c[j]);
+        }
+        continue;
       }
-      continue;
+      ++t;
+      ahead = stage[turn + (t & 31)];
+      if (op == I_NOP) continue;
+      if (op == I_SYNC) {
+        __syncthreads();
+        continue;
+      }
+      const S a = get(o.y);
+      if (op == I_OUTPUT) {
+        if (o.z && reduce) {   // reduced row z - 1: the instance's term, summed later
+          if (active) Wr[(long long)(o.z - 1) * ldr + i0] = a;
+        } else if (active) {
+          B* p = &Y[dst * ldy + i0];
+          *p = acc ? *p + (B)a : (B)a;
+        }
+        continue;
+      }
+      const S b = get(o.z), c = op >= I_MUL_ADD || op == FMA_CONST ? get(o.w) : S(0);
+      S r;
+      if (!MIXED || ((o.x >> 7) & 1u)) {
+        r = interp_op<S>(op, a, b, c);
+      } else {
+        r = (S)interp_op<float>(op, (float)a, (float)b, (float)c);
+      }
+      if (dst < n_shared) sm[dst * 32] = r;
+      else gm[(long long)(dst - n_shared) * ldw] = r;
     }
-    const S a = at(o.z), b = at(o.w);
-    const double kd = op == FMA_CONST ? K[aux] : 0.0;
-    S r;
-    if (!MIXED || ((o.x >> 7) & 1u)) {
-      r = eval_op<S>(op, a, b, (S)kd);
-    } else {
-      r = (S)eval_op<float>(op, (float)a, (float)b, (float)kd);
-    }
-    at(o.y) = r;
   }
 }
 
 template <typename B, typename S, bool MIXED>
-int launch(const IOp* ops, int64_t n_ops, const double* k, const void* X, int64_t ldx,
+int launch(const IOp* ops, const int32_t* begin, int ways, const void* k, const void* X, int64_t ldx,
            const void* X2, int64_t ldx2, int64_t split, void* Y, int64_t ldy, int64_t N, void* W,
            int64_t ldw, int64_t n_shared, int acc, int reduce, void* Wr, int64_t ldr,
            cudaStream_t st) {
   auto kern = interp_kernel<B, S, MIXED>;
-  size_t smem = (size_t)n_shared * kInterpBlock * sizeof(S);
+  const int groups = ways == 1 && (size_t)n_shared * 128 * sizeof(S) <= 160 * 1024 ? 4 : 1;   // per CTA
+  const size_t smem = (size_t)groups * ((size_t)n_shared * 32 * sizeof(S) + (size_t)ways * 64 * sizeof(uint4));
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
   }
-  long long grid = (N + kInterpBlock - 1) / kInterpBlock;
-  kern<<<(unsigned)grid, kInterpBlock, smem, st>>>(reinterpret_cast<const uint4*>(ops), n_ops, k,
-                                                    (const B*)X, ldx, (const B*)X2, ldx2, split, (B*)Y,
-                                                    ldy, N, (S*)W, ldw, (unsigned)n_shared, acc, reduce,
-                                                    (S*)Wr, ldr);
+  const long long grid = (N + 32 * groups - 1) / (32 * groups);
+  kern<<<(unsigned)grid, 32 * ways * groups, smem, st>>>(reinterpret_cast<const uint4*>(ops), begin, ways, (const S*)k,
+                                                (const B*)X, ldx, (const B*)X2, ldx2, split, (B*)Y,
+                                                ldy, N, (S*)W, ldw, (unsigned)n_shared, acc, reduce,
+                                                (S*)Wr, ldr);
   return (int)cudaGetLastError();
 }
 
@@ -199,21 +283,16 @@ __global__ void __launch_bounds__(512) sum_rows_kernel(const T* __restrict__ Y, 
 
 }  // namespace
 
-int interp_shared_slots(int dtype, int shared_kb) {
-  const size_t elt = dtype == CUSADI_F32 ? 4 : 8;
-  return (int)(((size_t)std::max(0, shared_kb) * 1024) / (kInterpBlock * elt));
-}
-
-int launch_interp(const IOp* ops, int64_t n_ops, const double* k, int dtype, const void* X,
+int launch_interp(const IOp* ops, const int32_t* begin, int ways, const void* k, int dtype, const void* X,
                   int64_t ldx, const void* X2, int64_t ldx2, int64_t split, void* Y, int64_t ldy,
                   int64_t N, void* W, int64_t ldw, int64_t n_shared, int acc, int reduce,
                   void* Wr, int64_t ldr, void* stream) {
   cudaStream_t st = (cudaStream_t)stream;
   if (dtype == CUSADI_F64)
-    return launch<double, double, false>(ops, n_ops, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
+    return launch<double, double, false>(ops, begin, ways, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
   if (dtype == CUSADI_F32)
-    return launch<float, float, false>(ops, n_ops, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
-  return launch<float, double, true>(ops, n_ops, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
+    return launch<float, float, false>(ops, begin, ways, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
+  return launch<float, double, true>(ops, begin, ways, k, X, ldx, X2, ldx2, split, Y, ldy, N, W, ldw, n_shared, acc, reduce, Wr, ldr, st);
 }
 
 // Dense copy of one sparse output argument: dense[k * ldd + i] = y[(off +

@@ -151,10 +151,11 @@ struct DevState {
   std::vector<CUmodule> mods;
   std::vector<CUfunction> fwd, adj;
   CUfunction adj_finish = nullptr;   // fixed-order sum of the reduced rows' per-instance terms
-  void* d_ops_fwd = nullptr;
-  double* d_k_fwd = nullptr;
-  void* d_ops_adj = nullptr;
-  double* d_k_adj = nullptr;
+  // interpreter streams and constants, [layout]: 0 Direction::ip, 1 ip_few
+  void* d_ops_fwd[2] = {};
+  double* d_k_fwd[2] = {};
+  void* d_ops_adj[2] = {};
+  double* d_k_adj[2] = {};
   int64_t* d_reduce_rows = nullptr;  // interpreter adjoint: rows summed over instances
   // host-buffer evaluation: a copy-in and a copy-out stream, one compute
   // stream per chunk, and the events that order them (created on first use)
@@ -171,7 +172,8 @@ struct Direction {
   std::vector<int64_t> hist, hist_f64;
   CodegenResult cg;
   std::vector<std::string> bins;
-  InterpProgram ip;
+  InterpProgram ip, ip_few;          // interpreter layouts: beyond kInterpFew instances, up to them
+  const InterpProgram& interp(int64_t N) const { return N <= kInterpFew ? ip_few : ip; }
 };
 
 }  // namespace
@@ -284,7 +286,7 @@ cusadi_status prepare_direction(cusadi_fn fn, Direction& d, bool adjoint) {
     fn->path = CUSADI_PATH_INTERP;
   }
   std::string err;
-  if (!pack_interp(d.g, d.ip, err, interp_shared_slots(fn->opt.dtype, fn->opt.interp_shared_kb)))
+  if (!pack_interp(d.g, d.ip, d.ip_few, err, fn->opt.dtype, fn->opt.interp_shared_kb))
     return fail(CUSADI_E_UNSUPPORTED, err);
   d.n_slots = d.ip.n_slots;
   return CUSADI_OK;
@@ -323,22 +325,34 @@ cusadi_status load_on_device(cusadi_fn fn, DevState& ds, bool adjoint) {
   }
   Direction& d = adjoint ? fn->adj : fn->fwd;
   if (fn->path == CUSADI_PATH_INTERP) {
-    void* ops = nullptr;
-    double* k = nullptr;
-    size_t ob = std::max<size_t>(d.ip.ops.size(), 1) * sizeof(IOp);
-    size_t kb = std::max<size_t>(d.ip.k.size(), 1) * sizeof(double);
-    if ((ce = cudaMalloc(&ops, ob)) != cudaSuccess) return cuda_fail("cudaMalloc", ce);
-    if ((ce = cudaMalloc((void**)&k, kb)) != cudaSuccess) { cudaFree(ops); return cuda_fail("cudaMalloc", ce); }
-    if (!d.ip.ops.empty()) cudaMemcpy(ops, d.ip.ops.data(), d.ip.ops.size() * sizeof(IOp), cudaMemcpyHostToDevice);
-    if (!d.ip.k.empty()) cudaMemcpy(k, d.ip.k.data(), d.ip.k.size() * sizeof(double), cudaMemcpyHostToDevice);
+    for (int v = 0; v < 2; ++v) {
+      const InterpProgram& ip = v ? d.ip_few : d.ip;
+      void* ops = nullptr;
+      double* k = nullptr;
+      // the streams, then the first instruction of each warp's
+      const size_t ob = ip.ops.size() * sizeof(IOp) + ip.begin.size() * sizeof(int32_t);
+      const size_t kb = std::max<size_t>(ip.k.size(), 1) * sizeof(double);
+      if ((ce = cudaMalloc(&ops, ob)) != cudaSuccess) return cuda_fail("cudaMalloc", ce);
+      if ((ce = cudaMalloc((void**)&k, kb)) != cudaSuccess) { cudaFree(ops); return cuda_fail("cudaMalloc", ce); }
+      (adjoint ? ds.d_ops_adj : ds.d_ops_fwd)[v] = ops;
+      (adjoint ? ds.d_k_adj : ds.d_k_fwd)[v] = k;
+      if (!ip.ops.empty()) cudaMemcpy(ops, ip.ops.data(), ip.ops.size() * sizeof(IOp), cudaMemcpyHostToDevice);
+      cudaMemcpy((IOp*)ops + ip.ops.size(), ip.begin.data(), ip.begin.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+      if (!ip.k.empty()) {                 // constants in the work slots' type
+        if (fn->opt.dtype == CUSADI_F32) {
+          const std::vector<float> kf(ip.k.begin(), ip.k.end());
+          cudaMemcpy(k, kf.data(), kf.size() * sizeof(float), cudaMemcpyHostToDevice);
+        } else {
+          cudaMemcpy(k, ip.k.data(), ip.k.size() * sizeof(double), cudaMemcpyHostToDevice);
+        }
+      }
+    }
     if (adjoint && !d.ip.reduce_rows.empty()) {
       const size_t rb = d.ip.reduce_rows.size() * sizeof(int64_t);
       if ((ce = cudaMalloc((void**)&ds.d_reduce_rows, rb)) != cudaSuccess) return cuda_fail("cudaMalloc", ce);
       cudaMemcpy(ds.d_reduce_rows, d.ip.reduce_rows.data(), rb, cudaMemcpyHostToDevice);
     }
     if ((ce = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail("upload", ce);
-    (adjoint ? ds.d_ops_adj : ds.d_ops_fwd) = ops;
-    (adjoint ? ds.d_k_adj : ds.d_k_fwd) = k;
   } else {
     std::vector<CUfunction>& fs = adjoint ? ds.adj : ds.fwd;
     fs.clear();
@@ -388,7 +402,7 @@ int64_t interp_ldw(int64_t N) { return round_up(std::max<int64_t>(N, 1), 128); }
 size_t direction_ws(cusadi_fn fn, const Direction& d, int64_t N) {
   if (N <= 0) return 0;
   if (fn->path == CUSADI_PATH_INTERP)   // global work slots (if any), then reduced-row terms
-    return ((size_t)d.ip.n_global * interp_ldw(N) +
+    return ((size_t)d.interp(N).n_global * interp_ldw(N) +
             d.ip.reduce_rows.size() * (size_t)round_up(N, 32)) * elt_ws(fn->opt.dtype);
   // rows carried between kernels, then (adjoint) one row of per-instance terms per reduced row
   return ((size_t)d.cg.ws_rows + d.cg.reduce_rows.size()) * round_up(N, 32) * elt_ws(fn->opt.dtype);
@@ -401,20 +415,21 @@ bool all_bcast(const Graph& g, int64_t rows) {
 }
 
 // ldw > 0: the workspace's leading dimension when W points into a larger
-// workspace (a chunk of a bigger batch); otherwise the one for N instances.
+// workspace (a chunk of a batch of n_total); otherwise the one for N instances.
 cusadi_status run(cusadi_fn fn, Direction& d, DevState& ds, bool adjoint, const void* X,
                   int64_t ldx, const void* X2, int64_t ldx2, void* Y, int64_t ldy, int64_t N,
-                  void* W, int acc, int reduce, cusadi_stream stream, int64_t ldw = 0) {
+                  void* W, int acc, int reduce, cusadi_stream stream, int64_t ldw = 0, int64_t n_total = 0) {
   if (fn->path == CUSADI_PATH_INTERP) {
-    const int64_t lw = ldw > 0 ? ldw : interp_ldw(N);
-    void* Wr = (W && !d.ip.reduce_rows.empty())
-                   ? (void*)((char*)W + (size_t)d.ip.n_global * lw *
-                                            elt_ws(fn->opt.dtype))
+    const int64_t lw = ldw > 0 ? ldw : interp_ldw(N), nt = n_total > 0 ? n_total : N;
+    const InterpProgram& ip = d.interp(nt);
+    const int v = &ip == &d.ip_few ? 1 : 0;
+    void* Wr = (W && !ip.reduce_rows.empty())
+                   ? (void*)((char*)W + (size_t)ip.n_global * lw * elt_ws(fn->opt.dtype))
                    : nullptr;
-    int rc = launch_interp((const IOp*)(adjoint ? ds.d_ops_adj : ds.d_ops_fwd),
-                           (int64_t)d.ip.ops.size(), adjoint ? ds.d_k_adj : ds.d_k_fwd,
+    const IOp* ops = (const IOp*)(adjoint ? ds.d_ops_adj : ds.d_ops_fwd)[v];
+    int rc = launch_interp(ops, (const int32_t*)(ops + ip.ops.size()), ip.ways, (adjoint ? ds.d_k_adj : ds.d_k_fwd)[v],
                            fn->opt.dtype, X, ldx, X2 ? X2 : X, ldx2, adjoint ? fn->ir.nnz_in : (int64_t)1 << 40,
-                           Y, ldy, N, W, lw, d.ip.n_shared, acc, reduce, Wr, round_up(N, 32), stream);
+                           Y, ldy, N, W, lw, ip.n_shared, acc, reduce, Wr, round_up(N, 32), stream);
     if (rc != 0) return fail(CUSADI_E_CUDA, std::string("interpreter launch: ") + cudaGetErrorString((cudaError_t)rc));
     return CUSADI_OK;
   }
@@ -622,10 +637,12 @@ void cusadi_free(cusadi_fn fn) {
     DevState& ds = kv.second;
     if (cudaSetDevice(kv.first) == cudaSuccess) {
       for (CUmodule m : ds.mods) if (driver().ok) driver().moduleUnload(m);
-      if (ds.d_ops_fwd) cudaFree(ds.d_ops_fwd);
-      if (ds.d_k_fwd) cudaFree(ds.d_k_fwd);
-      if (ds.d_ops_adj) cudaFree(ds.d_ops_adj);
-      if (ds.d_k_adj) cudaFree(ds.d_k_adj);
+      for (int v = 0; v < 2; ++v) {
+        if (ds.d_ops_fwd[v]) cudaFree(ds.d_ops_fwd[v]);
+        if (ds.d_k_fwd[v]) cudaFree(ds.d_k_fwd[v]);
+        if (ds.d_ops_adj[v]) cudaFree(ds.d_ops_adj[v]);
+        if (ds.d_k_adj[v]) cudaFree(ds.d_k_adj[v]);
+      }
       if (ds.d_reduce_rows) cudaFree(ds.d_reduce_rows);
       if (ds.h_in) cudaStreamDestroy(ds.h_in);
       if (ds.h_out) cudaStreamDestroy(ds.h_out);
@@ -876,7 +893,7 @@ cusadi_status cusadi_eval_host(cusadi_fn fn, const void* in_host, int64_t ld_in,
     if ((ce = cudaStreamWaitEvent(s_comp, ev_in, 0)) != cudaSuccess) return cuda_fail("cudaStreamWaitEvent", ce);
     void* wc = workspace ? (void*)((char*)workspace + (size_t)s0 * elt_ws(fn->opt.dtype)) : nullptr;
     st = run(fn, fn->fwd, *ds, false, din + (size_t)s0 * elt, N, nullptr, 0,
-             (char*)dev_out + (size_t)s0 * elt, N, n, wc, 0, 0, (cusadi_stream)s_comp, ldw);
+             (char*)dev_out + (size_t)s0 * elt, N, n, wc, 0, 0, (cusadi_stream)s_comp, ldw, N);
     if (st != CUSADI_OK) return st;
     if ((ce = cudaEventRecord(ev_comp, s_comp)) != cudaSuccess) return cuda_fail("cudaEventRecord", ce);
     if ((ce = cudaStreamWaitEvent(s_out, ev_comp, 0)) != cudaSuccess) return cuda_fail("cudaStreamWaitEvent", ce);
@@ -933,7 +950,7 @@ cusadi_status adjoint_impl(cusadi_fn fn, const void* in, int64_t ld_in, const vo
   // the kernels left each reduced row's per-instance terms in the workspace;
   // sum them in a fixed order (the same bits on every run)
   if (fn->path == CUSADI_PATH_INTERP) {
-    const InterpProgram& ip = fn->adj.ip;
+    const InterpProgram& ip = fn->adj.interp(N);
     const size_t off = (size_t)ip.n_global * interp_ldw(N) *
                        elt_ws(fn->opt.dtype);
     int rc = launch_reduce_finish(fn->opt.dtype, (char*)workspace + off, round_up(N, 32), N, ds->d_reduce_rows,
