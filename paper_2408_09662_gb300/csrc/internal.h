@@ -223,7 +223,7 @@ int launch_sum_rows(int dtype, const void* Y, int64_t ldy, int64_t rows, int64_t
                     int accumulate, void* stream);
 // dense copy of one output argument (kernels.cu); returns a cudaError_t value
 int launch_densify(int dtype, const void* y, int64_t ldy, int64_t off, const int32_t* map,
-                   int64_t n_dense, void* dense, int64_t ldd, int64_t N, int sms, void* stream);
+                   int64_t n_dense, void* dense, int64_t ldd, int64_t N, void* stream);
 
 // runtime.cpp: NVRTC compile with the in-memory and on-disk content-hash cache
 bool compile_nvrtc(const std::string& src, const std::string& name,

@@ -798,7 +798,7 @@ cusadi_status cusadi_densify(cusadi_fn fn, int arg, const void* y, int64_t ld_y,
       ds->dense_map[arg] = map;
     }
   }
-  int rc = launch_densify(fn->opt.dtype, y, ld_y, a.offset, map, n_dense, dense, ld_d, N, ds->sms, stream);
+  int rc = launch_densify(fn->opt.dtype, y, ld_y, a.offset, map, n_dense, dense, ld_d, N, stream);
   if (rc != 0) return fail(CUSADI_E_CUDA, std::string("densify launch: ") + cudaGetErrorString((cudaError_t)rc));
   return CUSADI_OK;
 }
