@@ -97,6 +97,7 @@ struct Gen {
   std::set<std::pair<int, bool>> calls2;       // (op, f64) of the paired (two-argument) versions
   bool own_f32 = false;                        // own FP32 sin/cos/exp used
   bool own_f64 = false;                        // FP64 math of math64.cuh used
+  std::set<std::string> wrappers;              // out-of-line wrappers of math64.cuh functions used
 
   Gen(const Graph& g_, const CodegenOptions& o_) : g(g_), o(o_) {}
 
@@ -151,6 +152,27 @@ int auto_register_cap(int64_t live) {
   const int64_t need = live + 20;
   if (need > 255) return 255;
   return need > 128 && need <= 168 ? 128 : 0;
+}
+
+// out-of-line forms of math64.cuh's functions with several results or arguments
+const char* const kRecip = "static __device__ __noinline__ cs_u64 cs_recip_d(double b) { return cs_recip64(b); }\n";
+const char* const kDivr = "static __device__ __noinline__ double cs_divr_d(double a, double b, cs_u64 r) "
+                          "{ return cs_divr64(a, b, r); }\n";
+const char* const kSincos = "static __device__ __noinline__ double2 cs_sincos_d(double x) "
+                            "{ double2 r; cs_sincos64(x, r.x, r.y); return r; }\n";
+
+// 2^64 / b of b's mantissa in [1, 2) (2^64 - 1 for 1), as cs_recip64 returns
+uint64_t recip_of(double b) {
+  uint64_t u;
+  std::memcpy(&u, &b, 8);
+  const uint64_t m = (u & 0xfffffffffffffull) | 1ull << 52;
+  if (m == 1ull << 52) return ~0ull;
+  return (uint64_t)(((unsigned __int128)1 << 116) / m);
+}
+// divisors that the constant form takes: normal, and inside cs_div_far's range
+bool const_divisor(const Node& b) {
+  const double m = std::fabs(b.k);
+  return b.op == CONST && m >= 0x1p-509 && m < 0x1p+513;
 }
 
 // the function itself, to be inlined where it is named
@@ -276,6 +298,14 @@ std::string op_expr(Gen& G, const Node& x, bool f, const std::string& A, const s
   if (f && own_f64_math(x.op)) {
     const int op = x.op == INV ? (int)DIV : (int)x.op;
     const bool inl = inlined(op, o.inline_math);
+    if (op == DIV && const_divisor(G.g.nodes[x.op == INV ? x.a : x.b])) {
+      const double b = G.g.nodes[x.op == INV ? x.a : x.b].k;
+      G.own_f64 = true;
+      if (!inl) G.wrappers.insert(kDivr);
+      char r[32];
+      std::snprintf(r, sizeof r, "0x%016" PRIx64 "ull", recip_of(b));
+      return std::string(inl ? "cs_divr64(" : "cs_divr_d(") + (x.op == INV ? One : A) + ", " + lit(b, true) + ", " + r + ")";
+    }
     if (!inl) G.calls.insert({op, true});
     G.own_f64 = true;
     return call_name(op, true, inl) + "(" + (x.op == INV ? One + ", " : "") + A + (x.op == DIV ? ", " + B : "") + ")";
@@ -500,11 +530,37 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   };
   std::vector<int64_t> partner(n, -1);
   std::vector<uint8_t> hoisted(n, 0);
+  // FP64 sin and cos of one argument: one call for both (the later one moves up
+  // to the earlier).  Divisors of at least three FP64 divisions of a segment: one
+  // reciprocal, then short divisions (math64.cuh).
+  const bool own64 = o.inline_math != 1;
+  std::vector<int64_t> trig(n, -1);            // per argument: its first sin or cos in the segment
+  std::vector<int32_t> n_div(n, 0);            // per divisor: divisions of the segment
+  std::vector<uint8_t> have_recip(n, 0);
+  auto divisor = [&](int64_t i) -> int32_t {
+    const Node& x = g.nodes[i];
+    if ((x.op != DIV && x.op != INV) || !G.node_f64((int32_t)i)) return -1;
+    const int32_t b = x.op == INV ? x.a : x.b;
+    return g.nodes[b].op == CONST || (spill && sp_kind[b] != SP_REG) ? -1 : b;
+  };
   for (int s = 0; s < nseg; ++s) {
     if (spill) spill_segment(s);
+    std::fill(trig.begin(), trig.end(), (int64_t)-1);
+    std::fill(n_div.begin(), n_div.end(), 0);
+    std::fill(have_recip.begin(), have_recip.end(), (uint8_t)0);
+    for (int64_t i = segs[s].first; own64 && i < segs[s].second; ++i) {
+      const Node& x = g.nodes[i];
+      if ((x.op == SIN || x.op == COS) && G.node_f64((int32_t)i) && g.nodes[x.a].op != CONST) {
+        const int64_t f = trig[x.a];
+        if (f < 0) trig[x.a] = i;
+        else if (g.nodes[f].op != x.op && partner[f] < 0) { partner[f] = i; hoisted[i] = 1; }
+      }
+      const int32_t b = divisor(i);
+      if (b >= 0) ++n_div[b];
+    }
     if (pairing) {
       for (int64_t i = segs[s].first; i < segs[s].second; ++i) {
-        if (!pairable(i) || hoisted[i]) continue;
+        if (!pairable(i) || hoisted[i] || partner[i] >= 0) continue;
         const int64_t lim = std::min<int64_t>(segs[s].second, i + 1 + o.pair_calls);
         for (int64_t j = i + 1; j < lim; ++j) {
           if (!pairable(j) || hoisted[j] || partner[j] >= 0 || g.nodes[j].op != g.nodes[i].op ||
@@ -525,6 +581,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     G.calls2.clear();
     G.own_f32 = false;
     G.own_f64 = false;
+    G.wrappers.clear();
     auto operand = [&](int32_t i, bool want_f64, int r) -> std::string {
       const Node& x = g.nodes[i];
       bool f = G.node_f64(i);
@@ -633,7 +690,19 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       const Node& x = g.nodes[i];
       const bool f = G.node_f64((int32_t)i);
       const char* T = G.ty(f);
-      if (pairing && partner[i] >= 0) {
+      const bool sincos = partner[i] >= 0 && g.nodes[partner[i]].op != x.op;
+      const int32_t dv = own64 ? divisor(i) : -1;
+      if (sincos) {
+        const int64_t j = partner[i];
+        G.own_f64 = true;
+        G.wrappers.insert(kSincos);
+        for (int l = 0; l < NL; ++l) {
+          const std::string A = operand(x.a, true, l);
+          body << "  const double2 p" << vname(i, l) << " = cs_sincos_d(" << A << ");\n"
+               << "  const double " << vname(i, l) << " = p" << vname(i, l) << (x.op == SIN ? ".x" : ".y") << ", "
+               << vname(j, l) << " = p" << vname(i, l) << (x.op == SIN ? ".y" : ".x") << ";\n";
+        }
+      } else if (pairing && partner[i] >= 0) {
         const int64_t j = partner[i];
         std::string A = operand(x.a, f, 0), Aj = operand(g.nodes[j].a, f, 0);
         G.calls2.insert({x.op, f});
@@ -642,7 +711,19 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
              << ", " << Aj << ");\n"
              << "  const " << T << " v" << i << " = p" << i << ".x;\n"
              << "  const " << T << " v" << j << " = p" << i << ".y;\n";
-      } else if (!(pairing && hoisted[i])) {    // a hoisted op was computed with its partner
+      } else if (dv >= 0 && n_div[dv] >= 3) {
+        G.own_f64 = true;
+        G.wrappers.insert(kRecip);
+        G.wrappers.insert(kDivr);
+        const bool shared = NL == 1 || (g.nodes[dv].op == INPUT && g.nodes[dv].bcast);
+        for (int l = 0; l < NL; ++l) {
+          const std::string A = x.op == INV ? "1.0" : operand(x.a, true, l), B = operand(dv, true, l);
+          const std::string r = "r" + std::to_string(dv) + (shared ? "" : "_" + std::to_string(l));
+          if (!have_recip[dv] && (l == 0 || !shared)) body << "  const cs_u64 " << r << " = cs_recip_d(" << B << ");\n";
+          body << "  const double " << vname(i, l) << " = cs_divr_d(" << A << ", " << B << ", " << r << ");\n";
+        }
+        have_recip[dv] = 1;
+      } else if (!hoisted[i]) {    // a hoisted op was computed with its partner
         for (int l = 0; l < NL; ++l) {
           std::string A = x.a >= 0 ? operand(x.a, f, l) : "";
           std::string B = x.b >= 0 ? operand(x.b, f, l) : "";
@@ -682,6 +763,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     if (NL > 1) src << kLaneAccess;
     if (G.own_f32) src << own_math_source(o.own_math);
     if (G.own_f64) src << kMath64Text;
+    for (const std::string& w : G.wrappers) src << w;
     if (o.debug_checks && !o.device_fn) src << "__device__ unsigned int cs_dbg;   // non-finite results\n";
     {
       for (auto& c : G.calls) {
@@ -929,6 +1011,7 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
     G.calls.clear();
     G.own_f32 = false;
     G.own_f64 = false;
+    G.wrappers.clear();
     const int nph_seg = segs[s].second - segs[s].first;
     // phase-major layout: every warp reaches the same __syncthreads() (aligned
     // barrier); a value used by its own warp in a later phase is declared once
@@ -1035,6 +1118,7 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
         << " warps per 32 instances, " << (segs[s].second - segs[s].first) << " phases\n";
     if (G.own_f32) src << own_math_source(o.own_math);
     if (G.own_f64) src << kMath64Text;
+    for (const std::string& w : G.wrappers) src << w;
     if (o.debug_checks && !o.device_fn) src << "__device__ unsigned int cs_dbg;   // non-finite results\n";
     {
       for (auto& c : G.calls) {

@@ -173,18 +173,23 @@ static __device__ __forceinline__ double cs_exp64(double x) {
   return __hiloint2double((int)((cs_hi32(n) >> 10) + (e << 20)), (int)__funnelshift_r((cs_u32)n, cs_hi32(n), 10));
 }
 
-// sin (quad = 0) or cos (quad = 1) of x, 2^-27 <= |x| < 2^18: |x| = k pi/2 + r,
-// |r| <= 0.82, r with lsb 2^-95 (a remainder below 2^-20 would keep too few bits:
-// library); 1 - sin(r)/r and 1 - cos r are polynomials in z = r^2 of degree 7
-// with coefficients by interpolation at Chebyshev nodes (gen_math64_tables.py),
+// sin and cos of x, 2^-27 <= |x| < 2^18: |x| = k pi/2 + r, |r| <= 0.82, r with
+// lsb 2^-95 (a remainder below 2^-20 would keep too few bits: library);
+// 1 - sin(r)/r and 1 - cos r are polynomials in z = r^2 of degree 7 with
+// coefficients by interpolation at Chebyshev nodes (gen_math64_tables.py),
 // evaluated as c1 - y (c2 - y (c3 - ...)), y = z/64, lsb 2^-61.
-static __device__ __forceinline__ double cs_sincos_d(double x, cs_u32 quad) {
-  const cs_u32 hi = (cs_u32)__double2hiint(x), lo = (cs_u32)__double2loint(x);
-  const cs_u32 ahi = hi & 0x7fffffffu;
+struct cs_trig {
+  cs_u32 nh, nl, lz;      // |r| = (nh:nl) 2^(-63 - lz), leading bit set
+  cs_u32 neg;             // bit 31: r negative
+  cs_u32 k;               // quadrant
+  cs_u64 z;               // r^2, lsb 2^-64
+  bool rare;
+};
+static __device__ __forceinline__ cs_trig cs_trig_reduce(cs_u32 hi, cs_u32 lo) {
+  cs_trig t;
+  const cs_u32 e = (hi & 0x7fffffffu) >> 20;
   const cs_u32 f3 = __funnelshift_l(lo, hi, 3);
-  const cs_u32 kb = __float_as_uint(fmaf(__uint_as_float(f3 + 0x40000000u), 0x1.45f306p-1f, 12582912.0f));
-  const cs_u32 k = kb - 0x4b400000u;
-  const cs_u32 e = ahi >> 20;
+  const cs_u32 k = __float_as_uint(fmaf(__uint_as_float(f3 + 0x40000000u), 0x1.45f306p-1f, 12582912.0f)) - 0x4b400000u;
   // |x| with lsb 2^-63 (words 1 and 2 of 96 bits) minus k pi/2
   const cs_u32 mh = (hi & 0xfffffu) | 0x100000u;
   const cs_u64 xw = cs_pack(__funnelshift_l(lo, mh, e - 1012u), lo << ((e - 1012u) & 31u));
@@ -193,80 +198,151 @@ static __device__ __forceinline__ double cs_sincos_d(double x, cs_u32 quad) {
   const cs_u64 d = xw - p1 - (cs_u64)((cs_u32)p0 != 0u);
   const cs_u32 s = (cs_u32)((int)cs_hi32(d) >> 31);                    // remainder negative: negate
   const cs_u32 r2 = cs_hi32(d) ^ s, r1 = (cs_u32)d ^ s, r0 = (0u - (cs_u32)p0) ^ s;
-  cs_u32 lz = (cs_u32)__clz((int)r2);
-  cs_u32 nh = __funnelshift_l(r1, r2, lz), nl = __funnelshift_l(r0, r1, lz);   // |r| = (nh:nl) 2^(-63 - lz)
-  cs_u32 neg = s;
-  const bool small = e < 1022u;                                        // |x| < 1/2: r = x
-  if (small) {
-    nh = __funnelshift_l(lo, hi, 11) | 0x80000000u;
-    nl = lo << 11;
-    lz = 1023u - e;
-    neg = 0u;
+  t.lz = (cs_u32)__clz((int)r2);
+  t.nh = __funnelshift_l(r1, r2, t.lz);
+  t.nl = __funnelshift_l(r0, r1, t.lz);
+  t.neg = s;
+  t.k = k;
+  t.rare = t.lz > 20u;
+  if (e < 1022u) {                                                     // |x| < 1/2: r = x
+    t.nh = __funnelshift_l(lo, hi, 11) | 0x80000000u;
+    t.nl = lo << 11;
+    t.lz = 1023u - e;
+    t.neg = t.k = 0u;
+    t.rare = false;
   }
-  if (lz > 20u && !small) return quad ? cs_cos_lib(x) : cs_sin_lib(x);
-  const cs_u64 rr = cs_shr64(cs_pack(nh, nl), lz - 1u);                // lsb 2^-64
+  const cs_u64 rr = cs_shr64(cs_pack(t.nh, t.nl), t.lz - 1u);          // lsb 2^-64
   const cs_u32 rh = cs_hi32(rr);
-  const cs_u64 z = cs_wide(rh, rh) + 2 * (cs_u64)__umulhi(rh, (cs_u32)rr);     // r^2, lsb 2^-64
+  t.z = cs_wide(rh, rh) + 2 * (cs_u64)__umulhi(rh, (cs_u32)rr);
+  return t;
+}
+// sin(r)/r (c false) or cos r (c true), lsb 2^-61
+static __device__ __forceinline__ cs_u64 cs_trig_poly(cs_u64 z, bool c) {
   const cs_u64 y = z >> 6;
   const cs_u32 yh = cs_hi32(y), yl = (cs_u32)y;
-  const cs_u32 kq = (small ? 0u : k) + quad;
-  const bool c = (kq & 1u) != 0u;
   const cs_u32 v6 = (c ? 0x47ba723fu : 0x0584834eu) - __umulhi(yh, c ? 0x18f9411cu : 0x01aab7f7u);   // lsb 2^-29
   cs_u64 v = (c ? 0x93f27bf8eedb71c8ull : 0x0d7322997086c494ull) - (cs_wide(yh, v6) + __umulhi(yl, v6));
   v = (c ? 0xd00d00ce5cd425faull : 0x171de3a53d560bf6ull) - cs_mul_top(y, v);
   v = (c ? 0xb60b60b60a9b65c4ull : 0x1a01a01a01947c49ull) - cs_mul_top(y, v);
   v = (c ? 0x555555555555338cull : 0x1111111111110f14ull) - cs_mul_top(y, v);
   v = (c ? 0x0fffffffffffffffull : 0x0555555555555555ull) - cs_mul_top(y, v);
-  const cs_u64 w = 0x2000000000000000ull - cs_mul_top(z, v);           // sin(r)/r or cos r, lsb 2^-61
-  if (c) { nh = 0x80000000u; nl = 0u; lz = 0u; neg = 0u; }
+  return 0x2000000000000000ull - cs_mul_top(z, v);
+}
+// (nh:nl) 2^(-63 - lz) w with the sign bit of sg, rounded
+static __device__ __forceinline__ double cs_trig_round(cs_u32 nh, cs_u32 nl, cs_u32 lz, cs_u64 w, cs_u32 sg) {
   const cs_u64 g = cs_mul_top(cs_pack(nh, nl), w << 2);                // lsb 2^-62, [0.66, 2)
   const cs_u32 h = 1u - (cs_hi32(g) >> 30);                            // leading bit to bit 62
   const cs_u64 n = (g << h) + 0x200u;
-  const cs_u32 sg = ((kq << 30) ^ neg ^ (quad ? 0u : hi)) & 0x80000000u;
-  return __hiloint2double((int)(((cs_hi32(n) >> 10) + ((1022u - lz - h) << 20)) | sg),
+  return __hiloint2double((int)(((cs_hi32(n) >> 10) + ((1022u - lz - h) << 20)) | (sg & 0x80000000u)),
                           (int)__funnelshift_r((cs_u32)n, cs_hi32(n), 10));
 }
+// |x| outside the range: too small (true) or for the library
+static __device__ __forceinline__ bool cs_trig_far(cs_u32 ahi) { return ahi - 0x3e400000u >= 0x41100000u - 0x3e400000u; }
 
+// sin (quad 0) or cos (quad 1)
+static __device__ __forceinline__ double cs_trig64(double x, cs_u32 quad) {
+  const cs_u32 hi = (cs_u32)__double2hiint(x), lo = (cs_u32)__double2loint(x);
+  cs_trig t = cs_trig_reduce(hi, lo);
+  if (t.rare) return quad ? cs_cos_lib(x) : cs_sin_lib(x);
+  const cs_u32 kq = t.k + quad;
+  const bool c = (kq & 1u) != 0u;
+  const cs_u64 w = cs_trig_poly(t.z, c);
+  if (c) { t.nh = 0x80000000u; t.nl = 0u; t.lz = 0u; t.neg = 0u; }
+  return cs_trig_round(t.nh, t.nl, t.lz, w, (kq << 30) ^ t.neg ^ (quad ? 0u : hi));
+}
 static __device__ __forceinline__ double cs_sin64(double x) {
   const cs_u32 ahi = (cs_u32)__double2hiint(x) & 0x7fffffffu;
-  if (ahi - 0x3e400000u >= 0x41100000u - 0x3e400000u) return ahi < 0x3e400000u ? x : cs_sin_lib(x);
-  return cs_sincos_d(x, 0u);
+  if (cs_trig_far(ahi)) return ahi < 0x3e400000u ? x : cs_sin_lib(x);
+  return cs_trig64(x, 0u);
 }
-
 static __device__ __forceinline__ double cs_cos64(double x) {
   const cs_u32 ahi = (cs_u32)__double2hiint(x) & 0x7fffffffu;
-  if (ahi - 0x3e400000u >= 0x41100000u - 0x3e400000u) return ahi < 0x3e400000u ? 1.0 : cs_cos_lib(x);
-  return cs_sincos_d(x, 1u);
+  if (cs_trig_far(ahi)) return ahi < 0x3e400000u ? 1.0 : cs_cos_lib(x);
+  return cs_trig64(x, 1u);
+}
+// both at once: one reduction, and the two polynomials overlap; the same bits
+static __device__ __forceinline__ void cs_sincos64(double x, double& sn, double& cs) {
+  const cs_u32 hi = (cs_u32)__double2hiint(x), lo = (cs_u32)__double2loint(x), ahi = hi & 0x7fffffffu;
+  if (cs_trig_far(ahi)) {
+    sn = ahi < 0x3e400000u ? x : cs_sin_lib(x);
+    cs = ahi < 0x3e400000u ? 1.0 : cs_cos_lib(x);
+    return;
+  }
+  const cs_trig t = cs_trig_reduce(hi, lo);
+  if (t.rare) { sn = cs_sin_lib(x); cs = cs_cos_lib(x); return; }
+  const bool odd = (t.k & 1u) != 0u;
+  // sin x: +-sin r (k even) or +-cos r; cos x the other, by quadrant k + 1
+  const cs_u32 ss = (t.k << 30) ^ hi, sc = (t.k + 1u) << 30;
+  const double a = cs_trig_round(t.nh, t.nl, t.lz, cs_trig_poly(t.z, false), t.neg ^ (odd ? sc : ss));
+  const double b = cs_trig_round(0x80000000u, 0u, 0u, cs_trig_poly(t.z, true), odd ? ss : sc);
+  sn = odd ? b : a;
+  cs = odd ? a : b;
 }
 
 // a / b, both magnitudes in [2^-509, 2^513): Y = 2^32/b from the single-precision
 // reciprocal, low by at most 2^-21.2 and never high (b is rounded up first and Y
-// lowered by 512), so that each quotient digit is low and each remainder positive
-// and exact modulo 2^64; the last remainder decides the rounding.
-static __device__ __forceinline__ double cs_div64(double a, double b) {
-  const cs_u32 ha = (cs_u32)__double2hiint(a), la = (cs_u32)__double2loint(a);
-  const cs_u32 hb = (cs_u32)__double2hiint(b), lb = (cs_u32)__double2loint(b);
-  if ((ha << 1) - 0x40400000u >= 0x7fc00000u || (hb << 1) - 0x40400000u >= 0x7fc00000u) {
-    const bool zero = ((ha & 0x7fffffffu) | la) == 0u;                 // 0 / normal
-    if (zero && (hb & 0x7fffffffu) - 0x00100000u < 0x7fe00000u) return __hiloint2double((int)((ha ^ hb) & 0x80000000u), 0);
-    return cs_div_lib(a, b);
-  }
-  const cs_u32 ah = (ha & 0xfffffu) | 0x100000u, bh = (hb & 0xfffffu) | 0x100000u;
-  const cs_u64 ma = cs_pack(ah, la), mb = cs_pack(bh, lb);
+// lowered by 512; checked for all 2^23 mantissas), so that each quotient digit is
+// low and each remainder positive and exact modulo 2^64; the last remainder
+// decides the rounding.
+static __device__ __forceinline__ bool cs_div_far(cs_u32 ha, cs_u32 hb) {   // outside the range
+  return (ha << 1) - 0x40400000u >= 0x7fc00000u || (hb << 1) - 0x40400000u >= 0x7fc00000u;
+}
+static __device__ __forceinline__ double cs_div_rare(double a, double b) {
+  const cs_u32 ha = (cs_u32)__double2hiint(a), la = (cs_u32)__double2loint(a), hb = (cs_u32)__double2hiint(b);
+  const bool zero = ((ha & 0x7fffffffu) | la) == 0u;                   // 0 / normal
+  if (zero && (hb & 0x7fffffffu) - 0x00100000u < 0x7fe00000u) return __hiloint2double((int)((ha ^ hb) & 0x80000000u), 0);
+  return cs_div_lib(a, b);
+}
+// 2^32/b for the mantissa of b as a number in [1, 2)
+static __device__ __forceinline__ cs_u32 cs_div_seed(cs_u32 hb, cs_u32 lb) {
   const float bf = __uint_as_float(((__funnelshift_l(lb, hb, 3) & 0x7fffffu) | 0x3f800000u) + 1u);
-  const cs_u32 Y = __float_as_uint(cs_rcpf(bf)) * 256u + (0x80000000u - 512u);
-  const cs_u32 q1 = __umulhi(__funnelshift_l(la, ah, 11), Y);          // lsb 2^-31
-  cs_u64 r = (ma << 31) - cs_mul_low(mb, q1);
-  const cs_u32 q2 = __umulhi(cs_hi32(r), Y);                           // lsb 2^-51
-  r = (r << 20) - cs_mul_low(mb, q2);
-  const cs_u32 q3 = __umulhi(cs_hi32(r), Y);                           // lsb 2^-71
-  const cs_u64 v = ((cs_wide(q1, 1u << 20) + q2) << 3) + (q3 >> 17);   // lsb 2^-54
+  return __float_as_uint(cs_rcpf(bf)) * 256u + (0x80000000u - 512u);
+}
+// rounds v, the quotient of the mantissas with lsb 2^-54 or up to one unit less
+static __device__ __forceinline__ double cs_div_round(cs_u64 v, cs_u32 ha, cs_u32 la, cs_u32 hb, cs_u64 mb) {
   const cs_u32 h = cs_hi32(v) >> 22;                                   // quotient >= 1
   cs_u64 t = v >> h;                                                   // 53 bits and the rounding bit, or one less
   const cs_u64 rem = cs_pack(la << (22u - h), 0u) - cs_mul_low(t, mb);
   t = (t + (rem >= mb ? 2u : 1u)) >> 1;
   const cs_u32 e = (ha & 0x7ff00000u) - (hb & 0x7ff00000u) + ((1021u + h) << 20);
   return __hiloint2double((int)((cs_hi32(t) + e) | ((ha ^ hb) & 0x80000000u)), (int)(cs_u32)t);
+}
+static __device__ __forceinline__ double cs_div64(double a, double b) {
+  const cs_u32 ha = (cs_u32)__double2hiint(a), la = (cs_u32)__double2loint(a);
+  const cs_u32 hb = (cs_u32)__double2hiint(b), lb = (cs_u32)__double2loint(b);
+  if (cs_div_far(ha, hb)) return cs_div_rare(a, b);
+  const cs_u32 ah = (ha & 0xfffffu) | 0x100000u, bh = (hb & 0xfffffu) | 0x100000u;
+  const cs_u64 ma = cs_pack(ah, la), mb = cs_pack(bh, lb);
+  const cs_u32 Y = cs_div_seed(hb, lb);
+  const cs_u32 q1 = __umulhi(__funnelshift_l(la, ah, 11), Y);          // lsb 2^-31
+  cs_u64 r = (ma << 31) - cs_mul_low(mb, q1);
+  const cs_u32 q2 = __umulhi(cs_hi32(r), Y);                           // lsb 2^-51
+  r = (r << 20) - cs_mul_low(mb, q2);
+  const cs_u32 q3 = __umulhi(cs_hi32(r), Y);                           // lsb 2^-71
+  return cs_div_round(((cs_wide(q1, 1u << 20) + q2) << 3) + (q3 >> 17), ha, la, hb, mb);
+}
+
+// Division by a divisor used several times: cs_recip64(b) is 2^64/b of its
+// mantissa, low by at most 4 units; the quotient of cs_divr64 then comes from one
+// product (low by less than 2^-60) and the same exact rounding: 38 instructions
+// in place of 75.  For constant divisors the compiler of the program provides r.
+static __device__ __forceinline__ cs_u64 cs_recip64(double b) {
+  const cs_u32 hb = (cs_u32)__double2hiint(b), lb = (cs_u32)__double2loint(b);
+  const cs_u64 mb = cs_pack((hb & 0xfffffu) | 0x100000u, lb);
+  const cs_u32 Y = cs_div_seed(hb, lb);
+  const cs_u32 q1 = __umulhi(0x80000000u, Y);                          // a = 1: lsb 2^-31
+  cs_u64 r = 0ull - cs_mul_low(mb, q1);                                // 2^83 modulo 2^64 is 0
+  const cs_u32 q2 = __umulhi(cs_hi32(r), Y);
+  r = (r << 20) - cs_mul_low(mb, q2);
+  const cs_u32 q3 = __umulhi(cs_hi32(r), Y);
+  return (cs_wide(q1, 1u << 20) << 13) + ((cs_u64)q2 << 13) + (q3 >> 7);
+}
+static __device__ __forceinline__ double cs_divr64(double a, double b, cs_u64 r) {
+  const cs_u32 ha = (cs_u32)__double2hiint(a), la = (cs_u32)__double2loint(a);
+  const cs_u32 hb = (cs_u32)__double2hiint(b), lb = (cs_u32)__double2loint(b);
+  if (cs_div_far(ha, hb)) return cs_div_rare(a, b);
+  const cs_u64 m = cs_pack(__funnelshift_l(la, ha, 11) | 0x80000000u, la << 11);
+  return cs_div_round(cs_mul_top(m, r) >> 9, ha, la, hb, cs_pack((hb & 0xfffffu) | 0x100000u, lb));
 }
 
 // sqrt(a) for normal a > 0: m = a 4^-h in [1, 4), Y = 2^32/sqrt(m) from the
