@@ -64,7 +64,7 @@ struct Ready {
   bool operator<(const Ready& o) const { return pri < o.pri || (pri == o.pri && i > o.i); }
 };
 
-CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost);
+CoopPlan plan_eft(const PhaseDag& d, int ways, double comm_cost);
 
 }  // namespace
 
@@ -162,15 +162,34 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
   d.deps.assign(n, {-1, -1, -1});
   d.skip.assign(n, 0);
   d.cost.assign(n, 0.0);
+  // a multiply whose only reader is an add or subtract goes with it, so that the
+  // compiler contracts the two as it does in the one-thread kernel
+  std::vector<int32_t> reads(n, 0), fused(n, -1);
+  for (const Node& x : g.nodes) {
+    if (x.a >= 0) ++reads[x.a];
+    if (x.b >= 0) ++reads[x.b];
+  }
+  for (int32_t o : g.out) ++reads[o];
   for (int64_t i = 0; i < n; ++i) {
-    if (is_leaf(g, i)) { d.skip[i] = 1; continue; }
     const Node& x = g.nodes[i];
+    if (is_leaf(g, i)) { d.skip[i] = 1; continue; }
+    if (x.op != ADD && x.op != SUB) continue;
+    for (int32_t m : {x.a, x.b})
+      if (fused[i] < 0 && (g.nodes[m].op == MUL || g.nodes[m].op == SQ) && reads[m] == 1 && g.nodes[m].f64 == x.f64) {
+        fused[i] = m;
+        d.skip[m] = 1;
+      }
+  }
+  for (int64_t i = 0; i < n; ++i) {
+    if (d.skip[i]) continue;
+    const Node& x = g.nodes[i];
+    const int32_t m = fused[i];
     d.cost[i] = op_cost(x, dtype);
-    if (x.a >= 0 && !is_leaf(g, x.a)) d.deps[i][0] = x.a;
-    if (x.b >= 0 && !is_leaf(g, x.b)) d.deps[i][1] = x.b;
+    const int32_t o[3] = {m < 0 ? x.a : g.nodes[m].a, m < 0 ? x.b : g.nodes[m].b, m < 0 ? -1 : (x.a == m ? x.b : x.a)};
+    for (int k = 0; k < 3; ++k) d.deps[i][k] = o[k] >= 0 && !is_leaf(g, o[k]) ? o[k] : -1;
   }
   d.finish();
-  CoopPlan best = plan_eft(g, ways, comm_cost, d.cost);
+  CoopPlan best = plan_eft(d, ways, comm_cost);
   double best_t = estimate_phases(d, best, barrier_cost(dtype));
   // FP64 phases hold as many ops at 13 times the cost
   const double unit = dtype == CUSADI_F64 ? 13.0 : 1.0;
@@ -179,29 +198,33 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
     const double t = estimate_phases(d, P, barrier_cost(dtype));
     if (t < best_t) { best_t = t; best = std::move(P); }
   }
+  for (int64_t i = 0; i < n; ++i)
+    if (fused[i] >= 0) {
+      best.owner[fused[i]] = best.owner[i];
+      best.phase[fused[i]] = best.phase[i];
+    }
   return best;
 }
 
 namespace {
 
-CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<double>& cost) {
-  const int64_t n = (int64_t)g.nodes.size();
+CoopPlan plan_eft(const PhaseDag& d, int ways, double comm_cost) {
+  const int64_t n = (int64_t)d.deps.size();
   CoopPlan P;
   P.ways = ways;
   P.owner.assign(n, -1);
   P.phase.assign(n, 0);
   std::vector<double> finish(n, 0.0), avail(ways, 0.0);
-  auto leaf = [&](int64_t i) { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; };
+  P.n_phases = 1;
   for (int64_t i = 0; i < n; ++i) {
-    if (leaf(i)) continue;
-    const Node& x = g.nodes[i];
+    if (d.skip[i]) continue;
     int best = 0;
     double best_f = 1e300;
     for (int w = 0; w < ways; ++w) {
       double start = avail[w];
-      for (int32_t o : {x.a, x.b})
-        if (o >= 0 && !leaf(o)) start = std::max(start, finish[o] + (P.owner[o] == w ? 0.0 : comm_cost));
-      double f = start + cost[i];
+      for (int32_t o : d.deps[i])
+        if (o >= 0) start = std::max(start, finish[o] + (P.owner[o] == w ? 0.0 : comm_cost));
+      const double f = start + d.cost[i];
       if (f < best_f - 1e-12 || (f < best_f + 1e-12 && avail[w] < avail[best])) {
         best = w;
         best_f = f;
@@ -211,13 +234,11 @@ CoopPlan plan_eft(const Graph& g, int ways, double comm_cost, const std::vector<
     finish[i] = best_f;
     avail[best] = best_f;
     int ph = 0;
-    for (int32_t o : {x.a, x.b})
-      if (o >= 0 && !leaf(o)) ph = std::max(ph, P.phase[o] + (P.owner[o] == best ? 0 : 1));
+    for (int32_t o : d.deps[i])
+      if (o >= 0) ph = std::max(ph, P.phase[o] + (P.owner[o] == best ? 0 : 1));
     P.phase[i] = ph;
+    P.n_phases = std::max(P.n_phases, ph + 1);
   }
-  P.n_phases = 1;
-  for (int64_t i = 0; i < n; ++i)
-    if (!leaf(i)) P.n_phases = std::max(P.n_phases, P.phase[i] + 1);
   return P;
 }
 
