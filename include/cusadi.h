@@ -91,7 +91,10 @@ typedef struct {
                                  (forward and adjoint kernels): `ways` warps split each
                                  program across a group of 32 instances (small batches,
                                  few-instance long programs; at large batches it can also
-                                 win: time it); 0: one instance per thread          (0) */
+                                 win: time it); 0: one instance per thread (an FP64
+                                 program of 64 to 6,000 ops, other launch options at
+                                 their defaults, runs as ways = 8 on as few instances as
+                                 the GPU holds at once that way: 4,864 to 19,456)   (0) */
   int32_t own_math;           /* FP32 sin/cos/exp: 0 the library's (out-of-line calls),
                                  1 the engine's own (<= 2 ulp) inlined, 2 the engine's
                                  own as out-of-line functions                      (0) */

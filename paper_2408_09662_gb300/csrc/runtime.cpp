@@ -145,11 +145,25 @@ const Driver& driver() {
 
 namespace {
 
+// Double-precision programs run few instances in their cooperative form although
+// ways = 0: as many groups of 32 as the GPU holds at once in that form, at most
+// kFewPerSm per SM.  An FP64 instruction holds its unit for 64 clocks whichever
+// warp issues it, so one thread per instance needs four warps per SM before an SM's
+// four units work at all.  One thread -> 8 warps per 32 instances, us: cart-pole N =
+// 1,000 22.6 -> 9.0, 9,000 22.6 -> 12.3, 19,000 22.6 -> 18.5; random 3,000 ops N =
+// 4,000 191 -> 45, 19,000 193 -> 99; SRB adjoint (one group per SM) N = 4,000 112 ->
+// 53.  Beyond, the two meet (cart-pole, N = 65,536: 59.5 and 61.5).  Programs above
+// kFewOps would pay for it in compile time.
+constexpr int64_t kFewMinOps = 64, kFewOps = 6000;
+constexpr int kFewWays = 8, kFewPerSm = 4;
+
 struct DevState {
   bool fwd_ready = false, adj_ready = false;
   int sms = 0;                       // streaming multiprocessors of the device
   std::vector<CUmodule> mods;
   std::vector<CUfunction> fwd, adj;
+  CUfunction fwd_few = nullptr, adj_few = nullptr;
+  int64_t fwd_few_n = 0, adj_few_n = 0;   // instances up to which those run
   CUfunction adj_finish = nullptr;   // fixed-order sum of the reduced rows' per-instance terms
   // interpreter streams and constants, [layout]: 0 Direction::ip, 1 ip_few
   void* d_ops_fwd[2] = {};
@@ -172,6 +186,8 @@ struct Direction {
   std::vector<int64_t> hist, hist_f64;
   CodegenResult cg;
   std::vector<std::string> bins;
+  CodegenResult cg_few;              // compiled path: cooperative form for at most kFew instances
+  std::string bin_few;               // (empty: none)
   InterpProgram ip, ip_few;          // interpreter layouts: beyond kInterpFew instances, up to them
   const InterpProgram& interp(int64_t N) const { return N <= kInterpFew ? ip_few : ip; }
 };
@@ -244,8 +260,19 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   } else {
     d.cg = generate(d.g, co);
   }
-  const size_t ns = d.cg.segs.size();
-  d.bins.assign(ns, std::string());
+  const cusadi_options& o = fn->opt;
+  if (o.dtype == CUSADI_F64 && o.ways == 0 && d.n_ops >= kFewMinOps && d.n_ops <= kFewOps &&
+      co.inst_per_thread <= 1 && co.sync_every == 0 && co.spill_values == 0 && co.pair_calls == 0 &&
+      co.maxrregcount == 0 && d.cg.segs.size() == 1) {
+    CodegenOptions cf = co;
+    cf.prefix = adjoint ? "cs_few_adj_f64" : "cs_few_f64";
+    cf.coop_groups = 1;
+    d.cg_few = generate_coop(d.g, cf, plan_coop(d.g, kFewWays, 8.0, o.dtype));
+    // the same workspace, so that calls take the same buffers
+    if (d.cg_few.segs.size() != 1 || d.cg_few.ws_rows != d.cg.ws_rows) d.cg_few = CodegenResult();
+  }
+  const size_t n_main = d.cg.segs.size(), ns = n_main + d.cg_few.segs.size();
+  d.bins.assign(n_main, std::string());
   std::vector<std::string> logs(ns);
   std::vector<uint8_t> ok(ns, 0);
   auto opts = nvrtc_options(fn->opt);
@@ -254,10 +281,11 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   nt = (int)std::min<size_t>((size_t)nt, ns);
   std::atomic<size_t> next{0};
   auto work = [&]() {
-    for (size_t s; (s = next.fetch_add(1)) < ns;)
-      ok[s] = compile_nvrtc(d.cg.segs[s].source, d.cg.segs[s].name, opts,
-                            fn->cache_dir.empty() ? nullptr : fn->cache_dir.c_str(), d.bins[s],
-                            logs[s]);
+    for (size_t s; (s = next.fetch_add(1)) < ns;) {
+      const Segment& seg = s < n_main ? d.cg.segs[s] : d.cg_few.segs[0];
+      ok[s] = compile_nvrtc(seg.source, seg.name, opts, fn->cache_dir.empty() ? nullptr : fn->cache_dir.c_str(),
+                            s < n_main ? d.bins[s] : d.bin_few, logs[s]);
+    }
   };
   if (nt <= 1) work();
   else {
@@ -267,7 +295,9 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   }
   if (injected("compile")) return fail(CUSADI_E_COMPILE, "NVRTC failure injected (CUSADI_INJECT=compile)");
   for (size_t s = 0; s < ns; ++s)
-    if (!ok[s]) return fail(CUSADI_E_COMPILE, "NVRTC failed on " + d.cg.segs[s].name + ": " + logs[s].substr(0, 4000));
+    if (!ok[s])
+      return fail(CUSADI_E_COMPILE, "NVRTC failed on " + (s < n_main ? d.cg.segs[s] : d.cg_few.segs[0]).name + ": " +
+                                        logs[s].substr(0, 4000));
   return CUSADI_OK;
 }
 
@@ -374,6 +404,21 @@ cusadi_status load_on_device(cusadi_fn fn, DevState& ds, bool adjoint) {
         if (r != CUDA_SUCCESS) return cuda_fail("cuModuleGetFunction", r);
       }
     }
+    if (!d.bin_few.empty()) {
+      CUmodule m;
+      CUresult r = driver().moduleLoadData(&m, d.bin_few.data());
+      if (r != CUDA_SUCCESS) return cuda_fail("cuModuleLoadData", r);
+      ds.mods.push_back(m);
+      CUfunction& f = adjoint ? ds.adj_few : ds.fwd_few;
+      r = driver().moduleGetFunction(&f, m, d.cg_few.segs[0].name.c_str());
+      if (r == CUDA_SUCCESS && d.cg_few.smem_bytes > 48 * 1024)
+        r = driver().funcSetAttribute(f, CU_FUNC_ATTRIBUTE_MAX_DYNAMIC_SHARED_SIZE_BYTES, (int)d.cg_few.smem_bytes);
+      int per_sm = 0;
+      if (r == CUDA_SUCCESS)
+        r = driver().occupancy(&per_sm, f, 32 * d.cg_few.coop_ways, (size_t)d.cg_few.smem_bytes);
+      if (r != CUDA_SUCCESS) return cuda_fail("cuModuleGetFunction", r);
+      (adjoint ? ds.adj_few_n : ds.fwd_few_n) = (int64_t)32 * ds.sms * std::min(per_sm, kFewPerSm);
+    }
   }
   (adjoint ? ds.adj_ready : ds.fwd_ready) = true;
   return CUSADI_OK;
@@ -464,6 +509,13 @@ cusadi_status run(cusadi_fn fn, Direction& d, DevState& ds, bool adjoint, const 
   }
   long long lx = ldx, lx2 = ldx2, ly = ldy, n = N, lw = ldw > 0 ? ldw : round_up(N, 32);
   const void* x2 = X2 ? X2 : X;
+  const CUfunction few = adjoint ? ds.adj_few : ds.fwd_few;
+  if (few && (n_total > 0 ? n_total : N) <= (adjoint ? ds.adj_few_n : ds.fwd_few_n)) {
+    void* args[] = {(void*)&X, &lx, (void*)&x2, &lx2, &Y, &ly, &n, &W, &lw, &acc, &reduce, &vec};
+    CUresult r = driver().launchKernel(few, (unsigned)((N + 31) / 32), 1, 1, 32u * (unsigned)d.cg_few.coop_ways, 1, 1,
+                                       (unsigned)d.cg_few.smem_bytes, (CUstream)stream, args, nullptr);
+    return r == CUDA_SUCCESS ? CUSADI_OK : cuda_fail("cuLaunchKernel", r);
+  }
   for (size_t s = 0; s < fs.size(); ++s) {
     void* args[] = {(void*)&X, &lx, (void*)&x2, &lx2, &Y, &ly, &n, &W, &lw, &acc, &reduce, &vec};
     CUresult r = driver().launchKernel(fs[s], grid, 1, 1, block, 1, 1, smem, (CUstream)stream, args, nullptr);

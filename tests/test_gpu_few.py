@@ -1,0 +1,49 @@
+"""Double-precision programs evaluated on few instances (as many groups of 32 as the
+GPU holds at once, one to four per SM) run in their cooperative form: same bits as
+ways = 8, same results as the one-thread form within the FP64 rule, on both sides
+of the limit, through every call that picks the form by the batch's size."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import Oracle, tolerance
+from paper_2408_09662_gb300 import inputs, programs
+from paper_2408_09662_gb300.api import Function
+
+pytestmark = pytest.mark.gpu
+
+FEW, MANY = 152 * 32, 4 * 152 * 32
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 1000, FEW, MANY + 1])
+def test_form_by_batch_size(n):
+    irb = programs.cartpole_rk4().to_bytes()
+    X = inputs.cartpole(n, seed=n)
+    x = torch.tensor(X, device="cuda")
+    fn = Function(irb, dtype="f64")
+    buf = torch.full((24, n + 7), 5.0, dtype=torch.float64, device="cuda")
+    y = fn(x, out=buf[:, :n])
+    same = Function(irb, dtype="f64", ways=8) if n <= FEW else Function(irb, dtype="f64", maxrregcount=128)
+    assert torch.equal(y, same(x))
+    assert torch.all(buf[:, n:] == 5.0)
+    orc = Oracle(irb)
+    ref = orc.eval(X)
+    assert np.all(np.abs(y.cpu().numpy() - ref) <= tolerance(orc, X, ref, 1e-12, kind=0))
+    host = fn.eval_host(torch.tensor(X).pin_memory(), chunks=3)     # the whole batch decides
+    assert torch.equal(host, y.cpu())
+
+
+def test_adjoint_with_shared_gradient():
+    irb = programs.srb_step().to_bytes()
+    n = 1000
+    rng = np.random.default_rng(4)
+    X = np.vstack([np.tile(rng.normal(0, 0.1, (144, 1)), (1, n)), rng.uniform(-0.1, 0.1, (12, n)), np.zeros((1, n))])
+    B = rng.standard_normal((13, n))
+    x, b = torch.tensor(X, device="cuda"), torch.tensor(B, device="cuda")
+    got = []
+    for fn in (Function(irb, dtype="f64"), Function(irb, dtype="f64", ways=8)):
+        g = torch.ones(157, dtype=torch.float64, device="cuda")
+        got.append((fn.adjoint(x, b, shared_out=g, accumulate_broadcast=True)[144:], g))
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    ref = Oracle(irb).adjoint(X, B)
+    np.testing.assert_allclose(got[0][1][:144].cpu().numpy() - 1.0, ref[:144].sum(1), rtol=1e-9, atol=1e-10)
