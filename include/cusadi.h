@@ -378,20 +378,20 @@ cusadi_status cusadi_densify(cusadi_fn fn, int arg, const void* y, int64_t ld_y,
  * with a persistent scheduler kernel.  Its CTAs repeatedly take the next tile
  * (one program, `block` consecutive instances) from an atomic ticket; tiles are
  * ordered longest program first, so the few-instance long programs start at
- * once and the short ones fill the GPU around them.  The launch (ticket reset +
- * kernel) is captured once per device in a CUDA graph and replayed.  The same
- * link also has one plain kernel per program (CUSADI_BATCH_PLAIN), so the two
- * modes run identical per-instance code and give bit-identical results.
+ * once and the short ones fill the GPU around them.  The buffers' addresses are
+ * a kernel argument.  The same link also has one plain kernel per program
+ * (CUSADI_BATCH_PLAIN), so the two modes run identical per-instance code and give
+ * bit-identical results.
  *
  * With ways = W > 1, programs with at most 8,192 instances and at least 20,000
  * ops (after the passes) become satellites: each is compiled on its own as a
  * cooperative kernel, W warps splitting the program over each group of 32
  * instances (parallelism inside one expression graph, which CusADi leaves to
- * future work, §VI), and the batch's graph runs them on parallel branches
- * beside the scheduler kernel, started first.  Such a long program with few
+ * future work, §VI), and a CUDA graph runs them on parallel branches beside
+ * the scheduler kernel, started first.  Such a long program with few
  * instances then stops setting the length of the launch.  Its plain mode
  * launches the same cooperative kernels. */
-#define CUSADI_BATCH_PERSISTENT 0  /* one graph launch: satellites + scheduler kernel */
+#define CUSADI_BATCH_PERSISTENT 0  /* scheduler kernel (with satellites: one graph launch) */
 #define CUSADI_BATCH_PLAIN 1       /* one kernel launch per program (segment), in order */
 
 /* Compiles and links n programs (irs[j] of nbytes[j] bytes) for N[j]
@@ -411,12 +411,11 @@ size_t cusadi_batch_workspace_bytes(cusadi_batch b);
  * [nnz_out_j x ld_out[j]] device buffers (ld >= N[j]) as for cusadi_eval.
  * mode: CUSADI_BATCH_PERSISTENT or CUSADI_BATCH_PLAIN.  The first call on a
  * device loads the modules and uploads the tile table (allocates; not
- * capturable); the first persistent call captures the graph.  Later calls
- * only copy the buffer table when it changed (a few hundred bytes; with
- * satellites the graph is then captured again, since their launches carry
- * the buffers' addresses) and launch.  The buffer table and the tile
- * counter belong to the batch (one per device), so calls on one batch must not
- * overlap on the GPU: issue them on one stream, or order them with events. */
+ * capturable); with satellites, a persistent call on other buffers than the last
+ * captures the graph again, since its launches carry the addresses.  Other
+ * calls only launch.  The tile counter belongs to the batch (one per device), so
+ * calls on one batch must not overlap on the GPU: issue them on one stream, or
+ * order them with events. */
 cusadi_status cusadi_batch_eval(cusadi_batch b, const void* const* in, const int64_t* ld_in,
                                 void* const* out, const int64_t* ld_out, void* workspace,
                                 int mode, cusadi_stream stream);

@@ -282,11 +282,11 @@ def tuned(program, x: torch.Tensor, dtype: str = "f64", candidates=(0, 2, 4), re
 
 class Batch:
     """Several programs, each over its own fixed instance count, evaluated by one
-    persistent kernel replayed from a CUDA graph (mode "persistent") or by one
-    plain kernel per program (mode "plain"); both run the same per-instance code.
-    With ways = W > 1, long programs with few instances run as cooperative
-    satellite kernels (W warps per group of 32 instances) beside the
-    persistent kernel, on parallel branches of the same graph."""
+    persistent kernel (mode "persistent") or by one plain kernel per program
+    (mode "plain"); both run the same per-instance code.  With ways = W > 1, long
+    programs with few instances run as cooperative satellite kernels (W warps per
+    group of 32 instances) beside the persistent kernel, on parallel branches of
+    a CUDA graph."""
 
     MODES = {"persistent": L.CUSADI_BATCH_PERSISTENT, "plain": L.CUSADI_BATCH_PLAIN}
 
@@ -330,7 +330,7 @@ class Batch:
 
     def workspace(self, device) -> torch.Tensor | None:
         """One workspace kept for the batch: calls on one batch must not overlap
-        on the GPU anyway (its buffer table and tile counter are shared)."""
+        on the GPU anyway (its tile counter is shared)."""
         nb = L.cusadi_batch_workspace_bytes(self._b)
         if nb == 0:
             return None

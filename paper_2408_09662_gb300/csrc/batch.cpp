@@ -5,10 +5,10 @@
 // instance count share one launch: each program is compiled as relocatable
 // one-instance device functions, linked with a scheduler kernel whose CTAs
 // take tiles (program, consecutive instances) from an atomic ticket in
-// longest-program-first order, and the launch is replayed from a CUDA graph.
-// Long programs with few instances ("satellites", with ways > 1) run instead
-// as cooperative kernels of their own, W warps per group of 32 instances, on
-// parallel branches of the same graph, started before the scheduler kernel.
+// longest-program-first order.  Long programs with few instances ("satellites",
+// with ways > 1) run instead as cooperative kernels of their own, W warps per
+// group of 32 instances, on parallel branches of a CUDA graph, started before
+// the scheduler kernel.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvJitLink.h>
@@ -50,6 +50,10 @@ struct BArg {
   long long ldw;
 };
 
+struct BArgs {
+  BArg a[kMaxProgs];
+};
+
 struct BatchProg {
   IRFile ir;
   Graph g;
@@ -82,8 +86,7 @@ struct BatchDev {
   int grid[kVariants] = {};
   void* d_tiles[kVariants] = {};
   unsigned* d_ticket = nullptr;
-  BArg* d_args = nullptr;
-  std::vector<BArg> last;
+  std::vector<BArg> last;                    // the buffers that exec[] carry
   cudaStream_t cap = nullptr;
   cudaGraphExec_t exec[kVariants] = {};
   bool captured = false;                     // exec[] hold the current buffers' launches
@@ -131,11 +134,13 @@ std::string scheduler_source(const cusadi_batch_s& b) {
       s << "extern \"C\" __device__ void " << seg.name << "(const " << T << "* __restrict__, long long, const "
         << T << "* __restrict__, long long, " << T << "* __restrict__, long long, " << TW
         << "* __restrict__, long long, long long);\n";
-  s << "static __device__ __forceinline__ void cs_run(const BArg* __restrict__ A, int p, long long i) {\n"
+  // the buffer table is a kernel argument, so other buffers cost no copy
+  s << "struct BArgs { BArg a[" << kMaxProgs << "]; };\n"
+    << "static __device__ __forceinline__ void cs_run(const BArgs& A, int p, long long i) {\n"
     << "  switch (p) {\n";
   for (size_t p = 0; p < b.progs.size(); ++p) {
     if (b.progs[p].sat) continue;
-    s << "    case " << p << ": {\n      const BArg a = A[" << p << "];\n";
+    s << "    case " << p << ": {\n      const BArg& a = A.a[" << p << "];\n";
     for (auto& seg : b.progs[p].cg.segs)
       s << "      " << seg.name << "(a.X, a.ldx, a.X, a.ldx, a.Y, a.ldy, a.W, a.ldw, i);\n";
     s << "      break;\n    }\n";
@@ -145,10 +150,12 @@ std::string scheduler_source(const cusadi_batch_s& b) {
     const int B = kBlocks[v];
     s << "extern \"C\" __global__ void __launch_bounds__(" << B << ") cs_batch_" << B
       << "(const BTile* __restrict__ tiles, int n_tiles, unsigned int* ticket,\n"
-      << "    const BArg* __restrict__ A) {\n"
+      << "    const __grid_constant__ BArgs A) {\n"
       << "  __shared__ int s_t;\n"
+      << "  // every CTA takes one ticket past the tiles: the last one wraps the counter to 0\n"
+      << "  const unsigned int wrap = (unsigned int)n_tiles + gridDim.x - 1u;\n"
       << "  for (;;) {\n"
-      << "    if (threadIdx.x == 0) s_t = (int)atomicAdd(ticket, 1u);\n"
+      << "    if (threadIdx.x == 0) s_t = (int)atomicInc(ticket, wrap);\n"
       << "    __syncthreads();\n"
       << "    const int t = s_t;\n"
       << "    __syncthreads();\n"
@@ -160,17 +167,17 @@ std::string scheduler_source(const cusadi_batch_s& b) {
   for (size_t p = 0; p < b.progs.size(); ++p) {
     if (b.progs[p].sat) continue;
     s << "extern \"C\" __global__ void __launch_bounds__(128) cs_plain_" << p
-      << "(const BArg* __restrict__ A, long long N) {\n"
+      << "(const __grid_constant__ BArgs A, long long N) {\n"
       << "  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;\n"
       << "  if (i < N) cs_run(A, " << p << ", i);\n}\n";
   }
   return s.str();
 }
 
-bool link(const std::vector<std::string>& objs, const cusadi_options& o, std::string& out,
+bool link(const std::vector<std::string>& objs, int maxrregcount, std::string& out,
           std::string& log) {
   std::vector<std::string> opts = {"-arch=sm_103a"};
-  if (o.maxrregcount > 0) opts.push_back("-maxrregcount=" + std::to_string(o.maxrregcount));
+  if (maxrregcount > 0) opts.push_back("-maxrregcount=" + std::to_string(maxrregcount));
   std::vector<const char*> c;
   for (auto& x : opts) c.push_back(x.c_str());
   nvJitLinkHandle h;
@@ -259,8 +266,7 @@ cusadi_status batch_device(cusadi_batch b, BatchDev** out) {
     }
   }
   if ((ce = cudaMalloc((void**)&d.d_ticket, 256)) != cudaSuccess) return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
-  if ((ce = cudaMalloc((void**)&d.d_args, kMaxProgs * sizeof(BArg))) != cudaSuccess)
-    return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
+  if ((ce = cudaMemset(d.d_ticket, 0, 256)) != cudaSuccess) return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
   if ((ce = cudaStreamCreateWithFlags(&d.cap, cudaStreamNonBlocking)) != cudaSuccess)
     return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
   if (b->n_sat > 0) {
@@ -299,20 +305,35 @@ cusadi_status launch_satellite(cusadi_batch b, BatchDev& d, size_t p, const BArg
   return CUSADI_OK;
 }
 
-// One graph per tile size: reset the ticket; fork the satellites onto side
-// streams (their kernels carry the buffers' addresses, so a change of buffers
-// re-captures); run the scheduler kernel; join.
+BArgs table(const std::vector<BArg>& args) {
+  BArgs t = {};
+  std::copy(args.begin(), args.end(), t.a);
+  return t;
+}
+
+// The scheduler kernel over variant v's tiles.
+cusadi_status launch_scheduler(cusadi_batch b, BatchDev& d, int v, const std::vector<BArg>& args, cudaStream_t st) {
+  int nt = (int)b->tiles[v].size();
+  if (nt == 0) return CUSADI_OK;
+  BArgs t = table(args);
+  void* kargs[] = {&d.d_tiles[v], &nt, &d.d_ticket, &t};
+  CUresult r = driver().launchKernel(d.persist[v], (unsigned)d.grid[v], 1, 1, (unsigned)kBlocks[v], 1, 1, 0u,
+                                     (CUstream)st, kargs, nullptr);
+  return r == CUDA_SUCCESS ? CUSADI_OK : bfail(CUSADI_E_CUDA, "cuLaunchKernel failed: " + std::to_string(r));
+}
+
+// With satellites, one graph per tile size: fork the satellites onto side
+// streams, run the scheduler kernel, join.  The launches carry the buffers'
+// addresses, so a change of buffers captures again.
 cusadi_status capture_graphs(cusadi_batch b, BatchDev& d, const std::vector<BArg>& args) {
   for (int v = 0; v < kVariants; ++v)
     if (d.exec[v]) { cudaGraphExecDestroy(d.exec[v]); d.exec[v] = nullptr; }
   d.captured = false;
-  const Driver& D = driver();
   for (int v = 0; v < kVariants; ++v) {
     cudaGraph_t g;
     cudaError_t ce = cudaStreamBeginCapture(d.cap, cudaStreamCaptureModeThreadLocal);
     if (ce != cudaSuccess) return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
-    bool ok = cudaMemsetAsync(d.d_ticket, 0, sizeof(unsigned), d.cap) == cudaSuccess;
-    if (b->n_sat > 0) ok = ok && cudaEventRecord(d.fork, d.cap) == cudaSuccess;
+    bool ok = cudaEventRecord(d.fork, d.cap) == cudaSuccess;
     std::vector<size_t> sats;                        // longest first
     for (size_t p = 0; p < b->progs.size(); ++p)
       if (b->progs[p].sat) sats.push_back(p);
@@ -326,16 +347,10 @@ cusadi_status capture_graphs(cusadi_batch b, BatchDev& d, const std::vector<BArg
            cudaEventRecord(d.join[k], d.side[k]) == cudaSuccess;
       ++k;
     }
-    int nt = (int)b->tiles[v].size();
-    CUresult r = CUDA_SUCCESS;
-    if (ok && nt > 0) {
-      void* kargs[] = {&d.d_tiles[v], &nt, &d.d_ticket, &d.d_args};
-      r = D.launchKernel(d.persist[v], (unsigned)d.grid[v], 1, 1, (unsigned)kBlocks[v], 1, 1, 0u,
-                         (CUstream)d.cap, kargs, nullptr);
-    }
+    ok = ok && launch_scheduler(b, d, v, args, d.cap) == CUSADI_OK;
     for (int j = 0; ok && j < k; ++j) ok = cudaStreamWaitEvent(d.cap, d.join[j], 0) == cudaSuccess;
     ce = cudaStreamEndCapture(d.cap, &g);
-    if (!ok || r != CUDA_SUCCESS || ce != cudaSuccess)
+    if (!ok || ce != cudaSuccess)
       return bfail(CUSADI_E_CUDA, "capturing the batch launch failed");
     ce = cudaGraphInstantiate(&d.exec[v], g, 0);
     cudaGraphDestroy(g);
@@ -417,6 +432,17 @@ cusadi_status cusadi_batch_create(const void* const* irs, const size_t* nbytes, 
   } catch (const std::bad_alloc&) {
     return bfail(CUSADI_E_OOM, "out of host memory");
   }
+  // Registers of the linked kernel.  Separate compilation gives it 254 whatever the
+  // programs need, 8 warps per SM; where the longest live set fits 128 or 168
+  // registers, ask for that: 16 or 12 warps (FP32 random programs of 300 to 5,000
+  // ops, 65,536 to 16,384 instances: 115 us at 254, 92 at 168, 106 at 128).
+  int cap = o.maxrregcount;
+  if (cap == 0) {
+    int64_t live = 0;
+    for (const BatchProg& P : b->progs)
+      if (!P.sat) live = std::max(live, max_live(P.g) * (o.dtype == CUSADI_F64 ? 2 : 1));
+    cap = live + 20 <= 128 ? 128 : (live + 20 <= 168 ? 168 : 0);
+  }
   // compile every segment (all programs) in parallel, then the scheduler, then link
   struct Job {
     const std::string* src; const std::string* name; std::string* bin; std::string log; bool ok;
@@ -437,10 +463,11 @@ cusadi_status cusadi_batch_create(const void* const* irs, const size_t* nbytes, 
   std::vector<std::string> opts = {"--gpu-architecture=sm_103a", "-std=c++17", "-lineinfo",
                                    "-DNDEBUG", "--relocatable-device-code=true"};
   opts.push_back(o.fmad ? "--fmad=true" : "--fmad=false");
-  if (o.maxrregcount > 0) opts.push_back("--maxrregcount=" + std::to_string(o.maxrregcount));
   std::vector<std::string> sopts;
   for (auto& x : opts)
     if (x != "--relocatable-device-code=true") sopts.push_back(x);
+  if (o.maxrregcount > 0) sopts.push_back("--maxrregcount=" + std::to_string(o.maxrregcount));
+  if (cap > 0) opts.push_back("--maxrregcount=" + std::to_string(cap));
   // biggest first, so the longest compile starts at once
   std::vector<size_t> order(jobs.size());
   std::iota(order.begin(), order.end(), 0);
@@ -466,7 +493,7 @@ cusadi_status cusadi_batch_create(const void* const* irs, const size_t* nbytes, 
   }
   objs.push_back(sched[0]);
   std::string log;
-  if (!link(objs, o, b->linked, log)) return bfail(CUSADI_E_COMPILE, "nvJitLink failed: " + log.substr(0, 4000));
+  if (!link(objs, cap, b->linked, log)) return bfail(CUSADI_E_COMPILE, "nvJitLink failed: " + log.substr(0, 4000));
   // tile tables, longest program first
   std::vector<int> byops(n);
   std::iota(byops.begin(), byops.end(), 0);
@@ -492,7 +519,6 @@ void cusadi_batch_free(cusadi_batch b) {
       if (d.d_tiles[v]) cudaFree(d.d_tiles[v]);
     }
     if (d.d_ticket) cudaFree(d.d_ticket);
-    if (d.d_args) cudaFree(d.d_args);
     if (d.cap) cudaStreamDestroy(d.cap);
     for (cudaStream_t st : d.side) cudaStreamDestroy(st);
     for (cudaEvent_t ev : d.join) cudaEventDestroy(ev);
@@ -537,25 +563,21 @@ cusadi_status cusadi_batch_eval(cusadi_batch b, const void* const* in, const int
   cusadi_status s = batch_device(b, &d);
   if (s != CUSADI_OK) return s;
   cudaStream_t st = (cudaStream_t)stream;
-  bool same = d->last.size() == n;
-  for (size_t p = 0; same && p < n; ++p) same = std::memcmp(&d->last[p], &args[p], sizeof(BArg)) == 0;
-  if (!same) {
-    // pageable source: the call returns once the bytes are staged, so `args` may go away
-    cudaError_t ce = cudaMemcpyAsync(d->d_args, args.data(), n * sizeof(BArg), cudaMemcpyHostToDevice, st);
-    if (ce != cudaSuccess) return bfail(CUSADI_E_CUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(ce));
-    d->last = args;
-    if (b->n_sat > 0) d->captured = false;   // the satellites' launches carry the addresses
-  }
   if (mode == CUSADI_BATCH_PERSISTENT) {
-    if (!d->captured) {
-      std::lock_guard<std::mutex> lk(b->mu);
+    if (b->n_sat == 0) return launch_scheduler(b, *d, b->variant, args, st);
+    std::lock_guard<std::mutex> lk(b->mu);
+    bool same = d->captured && d->last.size() == n;
+    for (size_t p = 0; same && p < n; ++p) same = std::memcmp(&d->last[p], &args[p], sizeof(BArg)) == 0;
+    if (!same) {
       s = capture_graphs(b, *d, args);
       if (s != CUSADI_OK) return s;
+      d->last = args;
     }
     cudaError_t ce = cudaGraphLaunch(d->exec[b->variant], st);
     if (ce != cudaSuccess) return bfail(CUSADI_E_CUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(ce));
     return CUSADI_OK;
   }
+  BArgs t = table(args);
   for (size_t p = 0; p < n; ++p) {
     if (b->progs[p].sat) {
       s = launch_satellite(b, *d, p, args[p], st);
@@ -563,7 +585,7 @@ cusadi_status cusadi_batch_eval(cusadi_batch b, const void* const* in, const int
       continue;
     }
     long long N = b->progs[p].N;
-    void* a[] = {&d->d_args, &N};
+    void* a[] = {&t, &N};
     CUresult r = driver().launchKernel(d->plain[p], (unsigned)((N + 127) / 128), 1, 1, 128, 1, 1, 0u,
                                        (CUstream)st, a, nullptr);
     if (r != CUDA_SUCCESS) return bfail(CUSADI_E_CUDA, "cuLaunchKernel failed: " + std::to_string(r));
