@@ -161,6 +161,9 @@ const char* const kDivr = "static __device__ __noinline__ double cs_divr_d(doubl
 const char* const kSincos = "static __device__ __noinline__ double2 cs_sincos_d(double x) "
                             "{ double2 r; cs_sincos64(x, r.x, r.y); return r; }\n";
 
+const char* const kSincosF = "static __device__ __noinline__ float2 cs_sincos_f(float x) "
+                             "{ float2 r; sincosf(x, &r.x, &r.y); return r; }\n";
+
 // FP32 division by a constant c > 0 without the compiler's range check and branch,
 // which keep it from overlapping one division with the next.  r is 1/c rounded to
 // nearest and the residual q c - x is exact, so one correction rounds x/c to
@@ -568,8 +571,8 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   };
   std::vector<int64_t> partner(n, -1);
   std::vector<uint8_t> hoisted(n, 0);
-  // FP64 sin and cos of one argument: one call for both (the later one moves up
-  // to the earlier).  Divisors of at least three FP64 divisions of a segment: one
+  // sin and cos of one argument: one call for both (the later one moves up to
+  // the earlier).  Divisors of at least three FP64 divisions of a segment: one
   // reciprocal, then short divisions (math64.cuh).
   const bool own64 = o.inline_math != 1;
   std::vector<int64_t> trig(n, -1);            // per argument: its first sin or cos in the segment
@@ -588,10 +591,11 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     std::fill(have_recip.begin(), have_recip.end(), (uint8_t)0);
     for (int64_t i = segs[s].first; own64 && i < segs[s].second; ++i) {
       const Node& x = g.nodes[i];
-      if ((x.op == SIN || x.op == COS) && G.node_f64((int32_t)i) && g.nodes[x.a].op != CONST) {
+      const bool f64 = G.node_f64((int32_t)i);
+      if ((x.op == SIN || x.op == COS) && (f64 || o.own_math == 0) && g.nodes[x.a].op != CONST) {
         const int64_t f = trig[x.a];
         if (f < 0) trig[x.a] = i;
-        else if (g.nodes[f].op != x.op && partner[f] < 0) { partner[f] = i; hoisted[i] = 1; }
+        else if (g.nodes[f].op != x.op && G.node_f64((int32_t)f) == f64 && partner[f] < 0) { partner[f] = i; hoisted[i] = 1; }
       }
       const int32_t b = divisor(i);
       if (b >= 0) ++n_div[b];
@@ -732,12 +736,12 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       const int32_t dv = own64 ? divisor(i) : -1;
       if (sincos) {
         const int64_t j = partner[i];
-        G.own_f64 = true;
-        G.wrappers.insert(kSincos);
+        if (f) G.own_f64 = true;
+        G.wrappers.insert(f ? kSincos : kSincosF);
         for (int l = 0; l < NL; ++l) {
-          const std::string A = operand(x.a, true, l);
-          body << "  const double2 p" << vname(i, l) << " = cs_sincos_d(" << A << ");\n"
-               << "  const double " << vname(i, l) << " = p" << vname(i, l) << (x.op == SIN ? ".x" : ".y") << ", "
+          const std::string A = operand(x.a, f, l);
+          body << "  const " << T << "2 p" << vname(i, l) << " = cs_sincos_" << (f ? "d(" : "f(") << A << ");\n"
+               << "  const " << T << " " << vname(i, l) << " = p" << vname(i, l) << (x.op == SIN ? ".x" : ".y") << ", "
                << vname(j, l) << " = p" << vname(i, l) << (x.op == SIN ? ".y" : ".x") << ";\n";
         }
       } else if (pairing && partner[i] >= 0) {
