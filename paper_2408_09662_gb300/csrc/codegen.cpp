@@ -547,6 +547,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     int64_t words = o.dtype == CUSADI_F64 ? 2 : 1;   // MIXED: most values are single
     cap = auto_register_cap(max_live(g) * words * NL);
   }
+  R.register_cap = cap;
   const bool clamped = o.adjoint || NL > 1 || (o.sync_every > 0 && !o.device_fn);
   R.inst_per_thread = NL;
   auto vname = [&](int64_t i, int r) {

@@ -102,6 +102,7 @@ struct CodegenResult {
   int coop_groups = 1;           // groups of 32 instances per CTA (cooperative kernels)
   int inst_per_thread = 1;       // consecutive instances per thread (one-thread kernels)
   int64_t smem_bytes = 0;        // dynamic shared memory per CTA (cooperative kernels)
+  int register_cap = 0;          // one-thread kernels: cap in the launch bounds (0: none)
 };
 
 struct CodegenOptions {

@@ -157,6 +157,14 @@ namespace {
 constexpr int64_t kFewMinOps = 64, kFewOps = 6000;
 constexpr int kFewWays = 8, kFewPerSm = 4;
 
+// Double-precision programs whose values exceed a thread's registers take 255, 8
+// warps per SM: fastest while the batch fits the GPU at once that way (38,912
+// instances).  Beyond, the same kernel at 128 registers keeps twice the warps in
+// flight for some more spills: N = 65,536, random 3,000 ops 433 -> 323 us, LDL^T n =
+// 22 514 -> 392, SRB adjoint 356 -> 346; N = 20,000 to 30,000 it is 5 % slower, and
+// so are programs above kFewOps (random 20,000 ops 3.39 -> 3.56 ms).
+constexpr int kManyCap = 128;
+
 struct DevState {
   bool fwd_ready = false, adj_ready = false;
   int sms = 0;                       // streaming multiprocessors of the device
@@ -164,6 +172,8 @@ struct DevState {
   std::vector<CUfunction> fwd, adj;
   CUfunction fwd_few = nullptr, adj_few = nullptr;
   int64_t fwd_few_n = 0, adj_few_n = 0;   // instances up to which those run
+  CUfunction fwd_many = nullptr, adj_many = nullptr;
+  int64_t fwd_many_n = 0, adj_many_n = 0; // instances beyond which those run
   CUfunction adj_finish = nullptr;   // fixed-order sum of the reduced rows' per-instance terms
   // interpreter streams and constants, [layout]: 0 Direction::ip, 1 ip_few
   void* d_ops_fwd[2] = {};
@@ -188,6 +198,8 @@ struct Direction {
   std::vector<std::string> bins;
   CodegenResult cg_few;              // compiled path: cooperative form for at most kFew instances
   std::string bin_few;               // (empty: none)
+  CodegenResult cg_many;             // compiled path: fewer registers for many instances
+  std::string bin_many;              // (empty: none)
   InterpProgram ip, ip_few;          // interpreter layouts: beyond kInterpFew instances, up to them
   const InterpProgram& interp(int64_t N) const { return N <= kInterpFew ? ip_few : ip; }
 };
@@ -271,8 +283,20 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
     // the same workspace, so that calls take the same buffers
     if (d.cg_few.segs.size() != 1 || d.cg_few.ws_rows != d.cg.ws_rows) d.cg_few = CodegenResult();
   }
-  const size_t n_main = d.cg.segs.size(), ns = n_main + d.cg_few.segs.size();
-  d.bins.assign(n_main, std::string());
+  if (o.dtype == CUSADI_F64 && o.ways == 0 && d.n_ops <= kFewOps && co.inst_per_thread <= 1 &&
+      co.sync_every == 0 && co.spill_values == 0 && d.cg.register_cap == 255 && d.cg.segs.size() == 1) {
+    CodegenOptions cm = co;
+    cm.prefix = adjoint ? "cs_many_adj_f64" : "cs_many_f64";
+    cm.maxrregcount = kManyCap;
+    d.cg_many = generate(d.g, cm);
+  }
+  struct Job { const Segment* seg; std::string* bin; };
+  std::vector<Job> jobs;
+  d.bins.assign(d.cg.segs.size(), std::string());
+  for (size_t s = 0; s < d.cg.segs.size(); ++s) jobs.push_back({&d.cg.segs[s], &d.bins[s]});
+  if (!d.cg_few.segs.empty()) jobs.push_back({&d.cg_few.segs[0], &d.bin_few});
+  if (!d.cg_many.segs.empty()) jobs.push_back({&d.cg_many.segs[0], &d.bin_many});
+  const size_t ns = jobs.size();
   std::vector<std::string> logs(ns);
   std::vector<uint8_t> ok(ns, 0);
   auto opts = nvrtc_options(fn->opt);
@@ -281,11 +305,9 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   nt = (int)std::min<size_t>((size_t)nt, ns);
   std::atomic<size_t> next{0};
   auto work = [&]() {
-    for (size_t s; (s = next.fetch_add(1)) < ns;) {
-      const Segment& seg = s < n_main ? d.cg.segs[s] : d.cg_few.segs[0];
-      ok[s] = compile_nvrtc(seg.source, seg.name, opts, fn->cache_dir.empty() ? nullptr : fn->cache_dir.c_str(),
-                            s < n_main ? d.bins[s] : d.bin_few, logs[s]);
-    }
+    for (size_t s; (s = next.fetch_add(1)) < ns;)
+      ok[s] = compile_nvrtc(jobs[s].seg->source, jobs[s].seg->name, opts,
+                            fn->cache_dir.empty() ? nullptr : fn->cache_dir.c_str(), *jobs[s].bin, logs[s]);
   };
   if (nt <= 1) work();
   else {
@@ -296,8 +318,7 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   if (injected("compile")) return fail(CUSADI_E_COMPILE, "NVRTC failure injected (CUSADI_INJECT=compile)");
   for (size_t s = 0; s < ns; ++s)
     if (!ok[s])
-      return fail(CUSADI_E_COMPILE, "NVRTC failed on " + (s < n_main ? d.cg.segs[s] : d.cg_few.segs[0]).name + ": " +
-                                        logs[s].substr(0, 4000));
+      return fail(CUSADI_E_COMPILE, "NVRTC failed on " + jobs[s].seg->name + ": " + logs[s].substr(0, 4000));
   return CUSADI_OK;
 }
 
@@ -419,6 +440,17 @@ cusadi_status load_on_device(cusadi_fn fn, DevState& ds, bool adjoint) {
       if (r != CUDA_SUCCESS) return cuda_fail("cuModuleGetFunction", r);
       (adjoint ? ds.adj_few_n : ds.fwd_few_n) = (int64_t)32 * ds.sms * std::min(per_sm, kFewPerSm);
     }
+    if (!d.bin_many.empty()) {
+      CUmodule m;
+      CUresult r = driver().moduleLoadData(&m, d.bin_many.data());
+      if (r != CUDA_SUCCESS) return cuda_fail("cuModuleLoadData", r);
+      ds.mods.push_back(m);
+      r = driver().moduleGetFunction(&(adjoint ? ds.adj_many : ds.fwd_many), m, d.cg_many.segs[0].name.c_str());
+      int per_sm = 0;
+      if (r == CUDA_SUCCESS) r = driver().occupancy(&per_sm, fs[0], fn->opt.block, 0);
+      if (r != CUDA_SUCCESS) return cuda_fail("cuModuleGetFunction", r);
+      (adjoint ? ds.adj_many_n : ds.fwd_many_n) = (int64_t)ds.sms * std::max(per_sm, 1) * fn->opt.block;
+    }
   }
   (adjoint ? ds.adj_ready : ds.fwd_ready) = true;
   return CUSADI_OK;
@@ -516,9 +548,11 @@ cusadi_status run(cusadi_fn fn, Direction& d, DevState& ds, bool adjoint, const 
                                        (unsigned)d.cg_few.smem_bytes, (CUstream)stream, args, nullptr);
     return r == CUDA_SUCCESS ? CUSADI_OK : cuda_fail("cuLaunchKernel", r);
   }
+  const CUfunction many = adjoint ? ds.adj_many : ds.fwd_many;
+  const bool use_many = many && (n_total > 0 ? n_total : N) > (adjoint ? ds.adj_many_n : ds.fwd_many_n);
   for (size_t s = 0; s < fs.size(); ++s) {
     void* args[] = {(void*)&X, &lx, (void*)&x2, &lx2, &Y, &ly, &n, &W, &lw, &acc, &reduce, &vec};
-    CUresult r = driver().launchKernel(fs[s], grid, 1, 1, block, 1, 1, smem, (CUstream)stream, args, nullptr);
+    CUresult r = driver().launchKernel(use_many ? many : fs[s], grid, 1, 1, block, 1, 1, smem, (CUstream)stream, args, nullptr);
     if (r != CUDA_SUCCESS) return cuda_fail("cuLaunchKernel", r);
   }
   return CUSADI_OK;

@@ -47,3 +47,24 @@ def test_adjoint_with_shared_gradient():
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
     ref = Oracle(irb).adjoint(X, B)
     np.testing.assert_allclose(got[0][1][:144].cpu().numpy() - 1.0, ref[:144].sum(1), rtol=1e-9, atol=1e-10)
+
+
+@pytest.mark.parametrize("n", [38912, 38913, 50001])
+def test_many_instances_at_128_registers(n):
+    """Values past a thread's registers: the 128-register form runs when the batch
+    no longer fits the GPU at 255.  The compiler may contract differently under
+    another register bound, so the bits are compared with contraction off."""
+    irb = programs.random_program(3000, seed=21).to_bytes()
+    X = inputs.normal(64, n, seed=2)
+    x = torch.tensor(X, device="cuda")
+    fn = Function(irb, dtype="f64", fmad=0)
+    y, b = fn(x), torch.tensor(inputs.normal(32, n, seed=3), device="cuda")
+    for cap in (128, 255):
+        other = Function(irb, dtype="f64", fmad=0, maxrregcount=cap)
+        assert torch.equal(y, other(x))
+    assert torch.equal(fn.adjoint(x, b), other.adjoint(x, b))
+    idx = np.arange(0, n, 997)
+    orc = Oracle(irb)
+    ref = orc.eval(X[:, idx])
+    got = Function(irb, dtype="f64")(x)[:, idx].cpu().numpy()
+    assert np.all(np.abs(got - ref) <= tolerance(orc, X[:, idx], ref, 1e-12, kind=0))
