@@ -158,6 +158,8 @@ int auto_register_cap(int64_t live) {
 const char* const kRecip = "static __device__ __noinline__ cs_u64 cs_recip_d(double b) { return cs_recip64(b); }\n";
 const char* const kDivr = "static __device__ __noinline__ double cs_divr_d(double a, double b, cs_u64 r) "
                           "{ return cs_divr64(a, b, r); }\n";
+const char* const kDivr2 = "static __device__ __noinline__ double2 cs_divr2_d(double a, double b, double d, cs_u64 r) "
+                           "{ double2 q; cs_divr64x2(a, b, d, r, q.x, q.y); return q; }\n";
 const char* const kSincos = "static __device__ __noinline__ double2 cs_sincos_d(double x) "
                             "{ double2 r; cs_sincos64(x, r.x, r.y); return r; }\n";
 
@@ -585,6 +587,20 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     const int32_t b = x.op == INV ? x.a : x.b;
     return g.nodes[b].op == CONST || (spill && sp_kind[b] != SP_REG) ? -1 : b;
   };
+  // a division by a reciprocal: its divisor's node (constants by node, too), else -1
+  const int64_t kDivPairWindow = 64;
+  std::vector<int64_t> waits(n, -1);           // division evaluated with a later one
+  std::vector<int64_t> first_use(n, INT64_MAX);
+  for (int64_t i = n - 1; i >= 0; --i)
+    for (int32_t a : {g.nodes[i].a, g.nodes[i].b})
+      if (a >= 0) first_use[a] = i;
+  auto short_div = [&](int64_t i) -> int32_t {
+    const Node& x = g.nodes[i];
+    if (G.leaf(i) || (x.op != DIV && x.op != INV) || !G.node_f64((int32_t)i)) return -1;
+    const int32_t b = x.op == INV ? x.a : x.b;
+    if (const_divisor(g.nodes[b])) return b;
+    return divisor(i) >= 0 && n_div[b] >= 3 ? b : -1;
+  };
   for (int s = 0; s < nseg; ++s) {
     if (spill) spill_segment(s);
     std::fill(trig.begin(), trig.end(), (int64_t)-1);
@@ -600,6 +616,21 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       }
       const int32_t b = divisor(i);
       if (b >= 0) ++n_div[b];
+    }
+    // two quotients by one divisor in one call: the later one moves up where its
+    // numerator is ready, else the earlier one waits where nothing needs it yet
+    for (int64_t i = segs[s].first; own64 && NL == 1 && !spill && i < segs[s].second; ++i) {
+      const int32_t b = short_div(i);
+      if (b < 0 || partner[i] >= 0 || hoisted[i] || waits[i] >= 0) continue;
+      const int64_t lim = std::min<int64_t>(segs[s].second, i + 1 + kDivPairWindow);
+      for (int64_t j = i + 1; j < lim; ++j) {
+        if (short_div(j) != b) continue;
+        const int32_t a = g.nodes[j].op == INV ? -1 : g.nodes[j].a;
+        const bool ready = a < 0 || G.leaf(a) || G.seg_of[a] != s || a < i;
+        if (ready) { partner[i] = j; hoisted[j] = 1; }
+        else if (first_use[i] > j) { partner[j] = i; waits[i] = j; }
+        if (ready || first_use[i] > j) break;
+      }
     }
     if (pairing) {
       for (int64_t i = segs[s].first; i < segs[s].second; ++i) {
@@ -727,15 +758,57 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
         for (int64_t r : G.out_rows[i]) store_out(r, v);
       }
     }
+    // where node i's value goes beside its register: spill slot, workspace row, outputs
+    auto keep = [&](int64_t i) {
+      const bool f = G.node_f64((int32_t)i);
+      if (spill && sp_kind[i] == SP_SMEM)
+        body << "  cs_sp[" << sp_idx[i] << " * blockDim.x] = (" << tw << ")v" << i << ";\n";
+      else if (spill && sp_kind[i] == SP_WS)
+        body << "  Wv[" << sp_idx[i] << "ll * ldw] = (" << tw << ")v" << i << ";\n";
+      if (G.ws_slot[i] >= 0) {
+        if (NL == 1) {
+          body << "  if (active) W[" << G.ws_slot[i] << "ll * ldw] = (" << tw << ")v" << i << ";\n";
+        } else {
+          body << "  if (active) cs_st" << NL << "(&W[" << G.ws_slot[i] << "ll * ldw], true, " << NL;
+          for (int l = 0; l < NL; ++l) body << ", (" << tw << ")" << vname(i, l);
+          body << ");\n";
+        }
+      }
+      if (!G.out_rows[i].empty()) {
+        std::vector<std::string> v = lane_values(i, f);
+        for (int64_t r : G.out_rows[i]) store_out(r, v);
+      }
+    };
     int64_t since_sync = 0;
     for (int64_t i = segs[s].first; i < segs[s].second; ++i) {
       if (G.leaf(i)) continue;
       const Node& x = g.nodes[i];
       const bool f = G.node_f64((int32_t)i);
       const char* T = G.ty(f);
-      const bool sincos = partner[i] >= 0 && g.nodes[partner[i]].op != x.op;
+      if (waits[i] >= 0) continue;   // evaluated with a later division
+      const bool two_div = partner[i] >= 0 && short_div(i) >= 0;
+      const bool sincos = partner[i] >= 0 && !two_div && g.nodes[partner[i]].op != x.op;
       const int32_t dv = own64 ? divisor(i) : -1;
-      if (sincos) {
+      if (two_div) {
+        const int64_t j = partner[i];
+        const int32_t b = short_div(i);
+        auto numerator = [&](int64_t k) { return g.nodes[k].op == INV ? std::string("1.0") : operand(g.nodes[k].a, true, 0); };
+        const std::string A = numerator(i), Aj = numerator(j), B = operand(b, true, 0);
+        G.own_f64 = true;
+        G.wrappers.insert(kDivr2);
+        std::string r = "r" + std::to_string(b);
+        if (g.nodes[b].op == CONST) {
+          char h[32];
+          std::snprintf(h, sizeof h, "0x%016" PRIx64 "ull", recip_of(g.nodes[b].k));
+          r = h;
+        } else if (!have_recip[b]) {
+          G.wrappers.insert(kRecip);
+          body << "  const cs_u64 " << r << " = cs_recip_d(" << B << ");\n";
+          have_recip[b] = 1;
+        }
+        body << "  const double2 p" << i << " = cs_divr2_d(" << A << ", " << Aj << ", " << B << ", " << r << ");\n"
+             << "  const double v" << i << " = p" << i << ".x, v" << j << " = p" << i << ".y;\n";
+      } else if (sincos) {
         const int64_t j = partner[i];
         if (f) G.own_f64 = true;
         G.wrappers.insert(f ? kSincos : kSincosF);
@@ -754,6 +827,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
              << ", " << Aj << ");\n"
              << "  const " << T << " v" << i << " = p" << i << ".x;\n"
              << "  const " << T << " v" << j << " = p" << i << ".y;\n";
+      } else if (hoisted[i]) {       // computed with its partner
       } else if (dv >= 0 && n_div[dv] >= 3) {
         G.own_f64 = true;
         G.wrappers.insert(kRecip);
@@ -766,30 +840,15 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
           body << "  const double " << vname(i, l) << " = cs_divr_d(" << A << ", " << B << ", " << r << ");\n";
         }
         have_recip[dv] = 1;
-      } else if (!hoisted[i]) {    // a hoisted op was computed with its partner
+      } else {
         for (int l = 0; l < NL; ++l) {
           std::string A = x.a >= 0 ? operand(x.a, f, l) : "";
           std::string B = x.b >= 0 ? operand(x.b, f, l) : "";
           body << "  const " << T << " " << vname(i, l) << " = " << op_expr(G, x, f, A, B, o) << ";\n";
         }
       }
-      if (spill && sp_kind[i] == SP_SMEM)
-        body << "  cs_sp[" << sp_idx[i] << " * blockDim.x] = (" << tw << ")v" << i << ";\n";
-      else if (spill && sp_kind[i] == SP_WS)
-        body << "  Wv[" << sp_idx[i] << "ll * ldw] = (" << tw << ")v" << i << ";\n";
-      if (G.ws_slot[i] >= 0) {
-        if (NL == 1) {
-          body << "  if (active) W[" << G.ws_slot[i] << "ll * ldw] = (" << tw << ")v" << i << ";\n";
-        } else {
-          body << "  if (active) cs_st" << NL << "(&W[" << G.ws_slot[i] << "ll * ldw], true, " << NL;
-          for (int l = 0; l < NL; ++l) body << ", (" << tw << ")" << vname(i, l);
-          body << ");\n";
-        }
-      }
-      if (!G.out_rows[i].empty()) {
-        std::vector<std::string> v = lane_values(i, f);
-        for (int64_t r : G.out_rows[i]) store_out(r, v);
-      }
+      keep(i);
+      if (two_div && waits[partner[i]] == i) keep(partner[i]);
       if (o.sync_every > 0 && !o.device_fn && ++since_sync >= o.sync_every) {
         body << "  __syncthreads();\n";
         since_sync = 0;

@@ -345,6 +345,23 @@ static __device__ __forceinline__ double cs_divr64(double a, double b, cs_u64 r)
   return cs_div_round(cs_mul_top(m, r) >> 9, ha, la, hb, cs_pack((hb & 0xfffffu) | 0x100000u, lb));
 }
 
+// two quotients by one divisor: their products and roundings overlap
+static __device__ __forceinline__ void cs_divr64x2(double a0, double a1, double b, cs_u64 r, double& q0, double& q1) {
+  const cs_u32 h0 = (cs_u32)__double2hiint(a0), l0 = (cs_u32)__double2loint(a0);
+  const cs_u32 h1 = (cs_u32)__double2hiint(a1), l1 = (cs_u32)__double2loint(a1);
+  const cs_u32 hb = (cs_u32)__double2hiint(b), lb = (cs_u32)__double2loint(b);
+  if (cs_div_far(h0, hb) || cs_div_far(h1, hb)) {
+    q0 = cs_div_far(h0, hb) ? cs_div_rare(a0, b) : cs_divr64(a0, b, r);
+    q1 = cs_div_far(h1, hb) ? cs_div_rare(a1, b) : cs_divr64(a1, b, r);
+    return;
+  }
+  const cs_u64 mb = cs_pack((hb & 0xfffffu) | 0x100000u, lb);
+  const cs_u64 v0 = cs_mul_top(cs_pack(__funnelshift_l(l0, h0, 11) | 0x80000000u, l0 << 11), r) >> 9;
+  const cs_u64 v1 = cs_mul_top(cs_pack(__funnelshift_l(l1, h1, 11) | 0x80000000u, l1 << 11), r) >> 9;
+  q0 = cs_div_round(v0, h0, l0, hb, mb);
+  q1 = cs_div_round(v1, h1, l1, hb, mb);
+}
+
 // sqrt(a) for normal a > 0: m = a 4^-h in [1, 4), Y = 2^32/sqrt(m) from the
 // single-precision reciprocal square root, low by at most 2^-20.4 and never high,
 // digits and exact remainders as for the division.
