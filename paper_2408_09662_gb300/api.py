@@ -31,6 +31,11 @@ def _program_bytes(program) -> bytes:
         return f.read()
 
 
+def _stream(t: torch.Tensor) -> int:
+    """The current stream of a CUDA tensor's device, as a pointer."""
+    return torch._C._cuda_getCurrentRawStream(t.get_device())
+
+
 class Function:
     """A straight-line program loaded into the engine.
 
@@ -61,6 +66,7 @@ class Function:
         self.inputs = [L.cusadi_arg_info(self._fn, False, j) for j in range(self.info.n_in)]
         self.outputs = [L.cusadi_arg_info(self._fn, True, j) for j in range(self.info.n_out)]
         self._stage = {}
+        self._no_ws = {}          # direction -> no batch size needs a workspace
 
     def __del__(self):
         if getattr(self, "_fn", None):
@@ -86,7 +92,13 @@ class Function:
         block to the current stream, so calls on different streams never share
         one (a single cached buffer would race between concurrent calls), and
         on the same stream the block is reused in stream order at no cost."""
-        nb = L.cusadi_workspace_bytes(self._fn, N, adjoint)
+        none = self._no_ws.get(adjoint)
+        if none is None:
+            # rows are a property of the program and, on the interpreter path, of
+            # its layout for few (up to 4,864) or many instances
+            none = self._no_ws[adjoint] = all(
+                L.cusadi_workspace_bytes(self._fn, n, adjoint) == 0 for n in (1, 1 << 20))
+        nb = 0 if none else L.cusadi_workspace_bytes(self._fn, N, adjoint)
         if nb == 0:
             return None
         return torch.empty(nb, dtype=torch.uint8, device=device)
@@ -97,6 +109,10 @@ class Function:
         return t.stride(0) if t.shape[0] > 1 else max(t.shape[1], 1)
 
     def _check(self, t: torch.Tensor, rows: int, name: str):
+        if t.is_cuda and t.dtype is self.torch_dtype and t.dim() == 2:
+            shape, stride = t.shape, t.stride()
+            if shape[0] == rows and stride[1] == 1:
+                return
         if not t.is_cuda:
             raise ValueError(f"{name} must be a CUDA tensor (data stays on the GPU)")
         if t.dtype != self.torch_dtype:
@@ -110,11 +126,11 @@ class Function:
         N = x.shape[1]
         if out is None:
             out = torch.empty((self.nnz_out, N), dtype=self.torch_dtype, device=x.device)
-        self._check(out, self.nnz_out, "out")
+        else:
+            self._check(out, self.nnz_out, "out")
         ws = self.workspace(N, False, x.device)
         L.cusadi_eval(self._fn, x.data_ptr(), self._ld(x), out.data_ptr(), self._ld(out), N,
-                      ws.data_ptr() if ws is not None else 0,
-                      torch.cuda.current_stream(x.device).cuda_stream)
+                      ws.data_ptr() if ws is not None else 0, _stream(x))
         return out
 
     def debug_count(self) -> int:
@@ -129,7 +145,7 @@ class Function:
         N = y.shape[1]
         d = torch.empty((a.nrow, a.ncol, N), dtype=self.torch_dtype, device=y.device)
         L.cusadi_densify(self._fn, arg, y.data_ptr(), self._ld(y), d.data_ptr(), max(N, 1), N,
-                         torch.cuda.current_stream(y.device).cuda_stream)
+                         _stream(y))
         return d
 
     def eval_host(self, x: torch.Tensor, out: torch.Tensor | None = None, chunks: int = 0,
@@ -189,7 +205,7 @@ class Function:
         flags = (L.CUSADI_ADJ_ACCUMULATE if accumulate else 0) | \
                 (L.CUSADI_ADJ_ACCUMULATE_BROADCAST if accumulate_broadcast else 0)
         ws = self.workspace(N, True, x.device)
-        stream = torch.cuda.current_stream(x.device).cuda_stream
+        stream = _stream(x)
         if shared_out is not None:
             if not shared_out.is_cuda or shared_out.dtype != self.torch_dtype or \
                     shared_out.numel() != self.nnz_in or not shared_out.is_contiguous():
@@ -221,8 +237,7 @@ def sum_instances(y: torch.Tensor, out: torch.Tensor | None = None,
     if not out.is_cuda or out.dtype != y.dtype or out.numel() != rows or not out.is_contiguous():
         raise ValueError("out must be a contiguous CUDA vector with one entry per row of y")
     dt = L.CUSADI_F64 if y.dtype == torch.float64 else L.CUSADI_F32
-    L.cusadi_sum_instances(dt, y.data_ptr(), Function._ld(y), rows, N, out.data_ptr(), accumulate,
-                           torch.cuda.current_stream(y.device).cuda_stream)
+    L.cusadi_sum_instances(dt, y.data_ptr(), Function._ld(y), rows, N, out.data_ptr(), accumulate, _stream(y))
     return out
 
 
@@ -348,8 +363,7 @@ class Batch:
         ws = self.workspace(dev)
         L.cusadi_batch_eval(self._b, [x.data_ptr() for x in xs], [Function._ld(x) for x in xs],
                             [o.data_ptr() for o in outs], [Function._ld(o) for o in outs],
-                            ws.data_ptr() if ws is not None else 0, self.MODES[mode],
-                            torch.cuda.current_stream(dev).cuda_stream)
+                            ws.data_ptr() if ws is not None else 0, self.MODES[mode], _stream(xs[0]))
         return outs
 
     def tune(self, xs, outs, reps: int = 5) -> int:
