@@ -162,8 +162,10 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
   d.deps.assign(n, {-1, -1, -1});
   d.skip.assign(n, 0);
   d.cost.assign(n, 0.0);
-  // a multiply whose only reader is an add or subtract goes with it, so that the
-  // compiler contracts the two as it does in the one-thread kernel
+  // An FP64 multiply whose only reader is an add or subtract goes with it, so that the
+  // compiler contracts the two as it does in the one-thread kernel: one instruction of
+  // the FP64 unit less.  Not in FP32, where the schedule matters more than the
+  // instruction (50,000 random ops, N = 8,192, 4 warps: 0.60 ms together, 0.45 apart).
   std::vector<int32_t> reads(n, 0), fused(n, -1);
   for (const Node& x : g.nodes) {
     if (x.a >= 0) ++reads[x.a];
@@ -175,7 +177,8 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
     if (is_leaf(g, i)) { d.skip[i] = 1; continue; }
     if (x.op != ADD && x.op != SUB) continue;
     for (int32_t m : {x.a, x.b})
-      if (fused[i] < 0 && (g.nodes[m].op == MUL || g.nodes[m].op == SQ) && reads[m] == 1 && g.nodes[m].f64 == x.f64) {
+      if (fused[i] < 0 && (g.nodes[m].op == MUL || g.nodes[m].op == SQ) && reads[m] == 1 &&
+          g.nodes[m].f64 == x.f64 && (dtype == CUSADI_F64 || (dtype == CUSADI_MIXED && x.f64))) {
         fused[i] = m;
         d.skip[m] = 1;
       }
