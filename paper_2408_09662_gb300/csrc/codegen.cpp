@@ -589,6 +589,11 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   };
   // a division by a reciprocal: its divisor's node (constants by node, too), else -1
   const int64_t kDivPairWindow = 64;
+  // FP32 sin and cos of one argument share a call when they are at most this far apart:
+  // a value kept longer costs a register (20,000 random ops, N = 16,384: 320 us
+  // whatever the distance, 316 at 64); pair_calls pairs calls in its own way (349 us
+  // at N = 65,536 and 128 registers, 378 with both).
+  const int64_t kSincosWindow = 64;
   std::vector<int64_t> waits(n, -1);           // division evaluated with a later one
   std::vector<int64_t> first_use(n, INT64_MAX);
   for (int64_t i = n - 1; i >= 0; --i)
@@ -609,9 +614,9 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     for (int64_t i = segs[s].first; own64 && i < segs[s].second; ++i) {
       const Node& x = g.nodes[i];
       const bool f64 = G.node_f64((int32_t)i);
-      if ((x.op == SIN || x.op == COS) && (f64 || o.own_math == 0) && g.nodes[x.a].op != CONST) {
+      if ((x.op == SIN || x.op == COS) && (f64 || (o.own_math == 0 && o.pair_calls == 0)) && g.nodes[x.a].op != CONST) {
         const int64_t f = trig[x.a];
-        if (f < 0) trig[x.a] = i;
+        if (f < 0 || (!f64 && i - f > kSincosWindow)) trig[x.a] = i;
         else if (g.nodes[f].op != x.op && G.node_f64((int32_t)f) == f64 && partner[f] < 0) { partner[f] = i; hoisted[i] = 1; }
       }
       const int32_t b = divisor(i);
