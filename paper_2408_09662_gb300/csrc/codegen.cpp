@@ -146,7 +146,7 @@ std::string launch_bounds(int threads, int maxrregcount) {
 //    the rest (LQR step, 510 live: 179 KB of spill stores at 32 registers and
 //    1.24 ms, 33 KB at 255; MPC mixed 1.65 -> 1.35 ms);
 //  * 129 to 168 would hold 12 warps per SM, at most 128 holds 16: cap 128 (FP32
-//    random 20k-op program at N = 65,536, 165 registers: 0.61 -> 0.37 ms; FP64
+//    random 20k-op program at N = 65,536, 165 registers: 0.61 -> 0.35 ms; FP64
 //    cart-pole, 138 registers: 0.075 -> 0.059 ms).
 int auto_register_cap(int64_t live) {
   const int64_t need = live + 20;
@@ -549,6 +549,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     int64_t words = o.dtype == CUSADI_F64 ? 2 : 1;   // MIXED: most values are single
     cap = auto_register_cap(max_live(g) * words * NL);
   }
+  cap = std::max(cap, 0);   // -1: none, and no rule either
   R.register_cap = cap;
   const bool clamped = o.adjoint || NL > 1 || (o.sync_every > 0 && !o.device_fn);
   R.inst_per_thread = NL;

@@ -163,6 +163,10 @@ constexpr int kFewWays = 8, kFewPerSm = 4;
 // flight for some more spills: N = 65,536, random 3,000 ops 433 -> 323 us, LDL^T n =
 // 22 514 -> 392, SRB adjoint 356 -> 346; N = 20,000 to 30,000 it is 5 % slower, and
 // so are programs above kFewOps (random 20,000 ops 3.39 -> 3.56 ms).
+// Single-precision and mixed programs that the compiler would give 129 to 168
+// registers do the same: their own count while the batch fits the GPU at once, where
+// a cap only adds spills (random 20,000 ops, N = 16,384: 312 against 333 us; 5,000 ops,
+// N = 32,768: 85 and 87), 128 beyond (20,000 ops, N = 65,536: 609 -> 351 us).
 constexpr int kManyCap = 128;
 
 struct DevState {
@@ -284,11 +288,21 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
     if (d.cg_few.segs.size() != 1 || d.cg_few.ws_rows != d.cg.ws_rows) d.cg_few = CodegenResult();
   }
   if (o.dtype == CUSADI_F64 && o.ways == 0 && d.n_ops <= kFewOps && co.inst_per_thread <= 1 &&
-      co.sync_every == 0 && co.spill_values == 0 && d.cg.register_cap == 255 && d.cg.segs.size() == 1) {
+      co.sync_every == 0 && co.spill_values == 0 && d.cg.register_cap == 255 && d.cg.segs.size() == 1 &&
+      co.maxrregcount == 0) {
     CodegenOptions cm = co;
     cm.prefix = adjoint ? "cs_many_adj_f64" : "cs_many_f64";
     cm.maxrregcount = kManyCap;
     d.cg_many = generate(d.g, cm);
+  } else if (o.dtype != CUSADI_F64 && o.ways == 0 && co.inst_per_thread <= 1 && co.sync_every == 0 &&
+             co.spill_values == 0 && co.maxrregcount == 0 && d.cg.register_cap == kManyCap &&
+             d.cg.segs.size() == 1) {
+    CodegenOptions cm = co;
+    cm.prefix = std::string(adjoint ? "cs_many_adj_" : "cs_many_") + tag[o.dtype];
+    cm.maxrregcount = kManyCap;
+    d.cg_many = generate(d.g, cm);
+    co.maxrregcount = -1;
+    d.cg = generate(d.g, co);
   }
   struct Job { const Segment* seg; std::string* bin; };
   std::vector<Job> jobs;

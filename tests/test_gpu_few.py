@@ -68,3 +68,14 @@ def test_many_instances_at_128_registers(n):
     ref = orc.eval(X[:, idx])
     got = Function(irb, dtype="f64")(x)[:, idx].cpu().numpy()
     assert np.all(np.abs(got - ref) <= tolerance(orc, X[:, idx], ref, 1e-12, kind=0))
+
+
+@pytest.mark.parametrize("n", [1, 45000, 65537])
+def test_single_precision_many_at_128_registers(n):
+    """FP32 programs of 129 to 168 registers: the compiler's count while the batch fits
+    the GPU at once, 128 beyond; the same bits on both sides (contraction off)."""
+    irb = programs.random_program(5000, seed=101).to_bytes()
+    x = torch.tensor(inputs.normal(64, n, seed=n), dtype=torch.float32, device="cuda")
+    fn = Function(irb, dtype="f32", fmad=0)
+    assert "__launch_bounds__(128) cs_fwd" in fn.source()
+    assert torch.equal(fn(x), Function(irb, dtype="f32", fmad=0, maxrregcount=128)(x))
