@@ -630,7 +630,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       if (b < 0 || partner[i] >= 0 || hoisted[i] || waits[i] >= 0) continue;
       const int64_t lim = std::min<int64_t>(segs[s].second, i + 1 + kDivPairWindow);
       for (int64_t j = i + 1; j < lim; ++j) {
-        if (short_div(j) != b) continue;
+        if (short_div(j) != b || partner[j] >= 0 || hoisted[j]) continue;   // in a pair already
         const int32_t a = g.nodes[j].op == INV ? -1 : g.nodes[j].a;
         const bool ready = a < 0 || G.leaf(a) || G.seg_of[a] != s || a < i;
         if (ready) { partner[i] = j; hoisted[j] = 1; }
