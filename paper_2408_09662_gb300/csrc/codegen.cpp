@@ -607,6 +607,11 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
     if (const_divisor(g.nodes[b])) return b;
     return divisor(i) >= 0 && n_div[b] >= 3 ? b : -1;
   };
+  // is node a's value there where node i is evaluated (a division that waits for a
+  // later one is not, whatever its index)
+  auto ready_at = [&](int32_t a, int64_t i, int s) {
+    return a < 0 || G.leaf(a) || G.seg_of[a] != s || (a < i && waits[a] < i);
+  };
   for (int s = 0; s < nseg; ++s) {
     if (spill) spill_segment(s);
     std::fill(trig.begin(), trig.end(), (int64_t)-1);
@@ -632,7 +637,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       for (int64_t j = i + 1; j < lim; ++j) {
         if (short_div(j) != b || partner[j] >= 0 || hoisted[j]) continue;   // in a pair already
         const int32_t a = g.nodes[j].op == INV ? -1 : g.nodes[j].a;
-        const bool ready = a < 0 || G.leaf(a) || G.seg_of[a] != s || a < i;
+        const bool ready = ready_at(a, i, s);
         if (ready) { partner[i] = j; hoisted[j] = 1; }
         else if (first_use[i] > j) { partner[j] = i; waits[i] = j; }
         if (ready || first_use[i] > j) break;
@@ -646,8 +651,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
           if (!pairable(j) || hoisted[j] || partner[j] >= 0 || g.nodes[j].op != g.nodes[i].op ||
               G.node_f64((int32_t)j) != G.node_f64((int32_t)i))
             continue;
-          const int32_t a = g.nodes[j].a;   // available at i: a leaf, carried in, or computed before i
-          if (!(G.leaf(a) || G.seg_of[a] != s || a < i)) continue;
+          if (!ready_at(g.nodes[j].a, i, s)) continue;
           partner[i] = j;
           hoisted[j] = 1;
           break;
