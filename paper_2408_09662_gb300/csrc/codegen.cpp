@@ -168,27 +168,28 @@ const char* const kSincosF = "static __device__ __noinline__ float2 cs_sincos_f(
 
 // FP32 division by a constant c > 0 without the compiler's range check and branch,
 // which keep it from overlapping one division with the next.  r is 1/c rounded to
-// nearest and the residual q c - x is exact, so one correction rounds x/c to
+// nearest and the residual q c - a is exact, so one correction rounds a/c to
 // nearest when q is within an ulp of it (P. Markstein, "Computation of elementary
 // functions on the IBM RISC System/6000 processor", 1990): |c r - 1| <= 2^-25 makes
-// it so; other constants take a correction more (cs_divc2_f).  Small x are scaled
-// by 2^64, or their residuals would underflow; a subnormal quotient is then rounded
-// twice (0.5000001 ulp).  Infinities and overflows keep the product.  Bits as
-// x / c.  SRB step FP32, 75 such divisions, N = 4,096: 7.1 -> 6.3 us, its adjoint 15.9
-// -> 13.3, N = 65,536: 10.3 -> 8.9 and 37.4 -> 30.7.
+// it so; other constants take a correction more (cs_divc2_f).  The quotient is
+// taken of a, x scaled up by 2^80 below 1 and down by 2^-64 from there, so that no
+// residual underflows and nothing overflows before the scale is undone; a subnormal
+// quotient is then rounded twice (0.5000001 ulp).  The residual of an infinite x is
+// a NaN, for which fminf puts a number that leaves the infinity.  Bits of x / c for
+// normal quotients.
 const char* const kDivc = R"(static __device__ __forceinline__ float cs_divc_f(float x, float c, float r) {
-  const bool t = fabsf(x) < 0x1p-60f;
-  const float a = t ? __fmul_rn(x, 0x1p+64f) : x, q = __fmul_rn(a, r), y = fmaf(fmaf(q, c, -a), -r, q);
-  const float z = fabsf(q) < __int_as_float(0x7f800000) ? y : q;
-  return t ? __fmul_rn(z, 0x1p-64f) : z;
+  const bool t = fabsf(x) < 1.0f;
+  const float a = __fmul_rn(x, t ? 0x1p+80f : 0x1p-64f), q = __fmul_rn(a, r);
+  const float y = fmaf(fminf(fmaf(q, c, -a), 0x1p+126f), -r, q);
+  return __fmul_rn(y, t ? 0x1p-80f : 0x1p+64f);
 }
 )";
 const char* const kDivc2 = R"(static __device__ __forceinline__ float cs_divc2_f(float x, float c, float r) {
-  const bool t = fabsf(x) < 0x1p-60f;
-  const float a = t ? __fmul_rn(x, 0x1p+64f) : x, q = __fmul_rn(a, r), p = fmaf(fmaf(q, c, -a), -r, q),
-              y = fmaf(fmaf(p, c, -a), -r, p);
-  const float z = fabsf(q) < __int_as_float(0x7f800000) ? y : q;
-  return t ? __fmul_rn(z, 0x1p-64f) : z;
+  const bool t = fabsf(x) < 1.0f;
+  const float a = __fmul_rn(x, t ? 0x1p+80f : 0x1p-64f), q = __fmul_rn(a, r);
+  const float p = fmaf(fminf(fmaf(q, c, -a), 0x1p+126f), -r, q);
+  const float y = fmaf(fminf(fmaf(p, c, -a), 0x1p+126f), -r, p);
+  return __fmul_rn(y, t ? 0x1p-80f : 0x1p+64f);
 }
 )";
 
