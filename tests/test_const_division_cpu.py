@@ -7,7 +7,7 @@ from paper_2408_09662_gb300 import tracer as T
 from paper_2408_09662_gb300.api import Function
 
 CONSTANTS = [k / 1000 for k in range(1, 1000) if k not in (125, 250, 500)] + [
-    3.0, 5.0, 6.0, 7.0, 10.0, 12.0, 24.0, 49.0, 1.0000001, 1.9999999, 8388609.0, 16777215.0, 1e10, 1.1 * 2.0 ** -40]
+    3.0, 5.0, 6.0, 7.0, 10.0, 12.0, 24.0, 49.0, 1.0000001, 1.9999999, 8388609.0, 16777215.0, 16777214.0, 1.1 * 2.0 ** -20]
 
 HOST = r"""
 #include <cmath>
@@ -24,14 +24,14 @@ static float __int_as_float(int i) { return as<float>(i); }
 static u32 __float_as_uint(float f) { return as<u32>(f); }
 static float __uint_as_float(u32 u) { return as<float>(u); }
 FUNCTIONS
-static const struct { int two; float c, r; } cs[] = { TABLE };
+static const struct { float c; float (*divide)(float); } cs[] = { TABLE };
 static std::mt19937_64 g(1);
 int main() {
   for (auto& k : cs) {
     long bad = 0;
     float at = 0;
     auto check = [&](float x) {
-      const float y = k.two ? cs_divc2_f(x, k.c, k.r) : cs_divc_f(x, k.c, k.r), w = x / k.c;
+      const float y = k.divide(x), w = x / k.c;
       if (as<u32>(y) != as<u32>(w) && !(std::isnan(y) && std::isnan(w))) { ++bad; at = x; }
     };
     ARGUMENTS
@@ -53,10 +53,11 @@ def differences(tmp_path, arguments):
     ir = T.Function([("x", [x])], [("y", [x / c for c in CONSTANTS])]).to_ir()
     src = Function(ir, dtype="f32", cache_dir=None).source()
     functions = re.findall(r"static __device__ __forceinline__ float cs_divc2?_f\(.*?\n}\n", src, flags=re.S)
-    calls = re.findall(r"cs_divc(2?)_f\(v\d+, \((\S+?f)\), \((\S+?f)\)\);", src)
-    assert len(functions) == 2 and len(calls) == len(CONSTANTS) and len({c[0] for c in calls}) == 2
+    calls = re.findall(r" (cs_divc2?_f)\(v\d+, (\S+), (.*)\);", src)
+    assert len(calls) == len(CONSTANTS) and len({c[0] for c in calls}) == 2
     text = HOST.replace("FUNCTIONS", "".join(functions)).replace("ARGUMENTS", arguments)
-    text = text.replace("TABLE", ", ".join(f"{{{1 if two else 0}, {c}, {r}}}" for two, c, r in calls))
+    text = text.replace("TABLE", ", ".join(
+        f"{{{c}, [](float x) {{ return {f}(x, {c}, {rest}); }}}}" for f, c, rest in calls))
     (tmp_path / "host.cpp").write_text(text)
     exe = str(tmp_path / "host")
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-o", exe, str(tmp_path / "host.cpp")], check=True)
@@ -66,3 +67,14 @@ def differences(tmp_path, arguments):
 def test_normal_quotients_and_overflow(tmp_path):
     arguments = OVERFLOW + EVERY_EXPONENT.replace("KEEP", "std::fabs((double)x / k.c) >= 0x1p-126")
     assert differences(tmp_path, arguments) == ""
+
+
+# x whose quotients are subnormal: every exponent, and next to halves of the grid
+SUBNORMAL = ("for (int i = 0; i < 4000; ++i) { const double h = ((double)(g() % (1u << (1 + g() % 23))) + 0.5) * 0x1p-149;"
+             "  const float x = (float)(h * k.c); check(x); check(-std::nextafterf(x, 1)); check(std::nextafterf(x, -1)); }"
+             "for (int i = 0; i < 4000; ++i) check(as<float>((u32)(g() % as<u32>(std::fmax(k.c, 0x1p-20f) * 0x1p-125f))));"
+             "for (u32 i = 0; i < 3000; ++i) check(as<float>(i));")
+
+
+def test_subnormal_quotients(tmp_path):
+    assert differences(tmp_path, SUBNORMAL + EVERY_EXPONENT.replace("KEEP", "true")) == ""

@@ -39,3 +39,23 @@ def test_division_by_constants_rounds_to_nearest(ways):
             zero = want == 0
             np.testing.assert_array_equal(np.signbit(y[k][zero]), np.signbit(want[zero]), err_msg=str(c))
             assert np.all(np.abs(y[k][sub].astype(np.float64) - want[sub]) <= 2.0 ** -149), c
+
+
+@pytest.mark.parametrize("ways", [0, 2])
+def test_division_by_constants_at_both_ends_of_the_range(ways):
+    """Subnormal quotients, and quotients next to overflow: the bits of x / c."""
+    (x,) = T.Graph().symbols(1)
+    ir = T.Function([("x", [x])], [("y", [x / c for c in CONSTANTS])]).to_ir()
+    rng = np.random.default_rng(4)
+    c = np.abs(np.array(CONSTANTS))
+    half = (rng.integers(0, 1 << 23, 1 << 14) + 0.5) * 2.0 ** -149
+    near = (half[:, None] * c).astype(np.float32).ravel()
+    top = np.minimum(c * 2.0 ** 128, 3.4028234e38).astype(np.float32)
+    X = np.concatenate([near, np.nextafter(near, np.float32(0)), -near, np.arange(1 << 16, dtype=np.uint32).view(np.float32)]
+                       + [(top.view(np.int32) + np.int32(i)).view(np.float32) for i in range(-32, 33)])
+    y = Function(ir, dtype="f32", ways=ways)(torch.tensor(X[None], device="cuda")).cpu().numpy()
+    with np.errstate(all="ignore"):
+        for k, v in enumerate(CONSTANTS):
+            want = X / np.float32(v)
+            same = (y[k].view(np.uint32) == want.view(np.uint32)) | (np.isnan(y[k]) & np.isnan(want))
+            assert np.all(same), (v, X[~same][:3])
