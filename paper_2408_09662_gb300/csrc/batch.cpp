@@ -151,15 +151,15 @@ std::string scheduler_source(const cusadi_batch_s& b) {
     s << "extern \"C\" __global__ void __launch_bounds__(" << B << ") cs_batch_" << B
       << "(const BTile* __restrict__ tiles, int n_tiles, unsigned int* ticket,\n"
       << "    const __grid_constant__ BArgs A) {\n"
-      << "  __shared__ int s_t;\n"
+      << "  __shared__ unsigned int s_t;\n"
       << "  // every CTA takes one ticket past the tiles: the last one wraps the counter to 0\n"
       << "  const unsigned int wrap = (unsigned int)n_tiles + gridDim.x - 1u;\n"
       << "  for (;;) {\n"
-      << "    if (threadIdx.x == 0) s_t = (int)atomicInc(ticket, wrap);\n"
+      << "    if (threadIdx.x == 0) s_t = atomicInc(ticket, wrap);\n"
       << "    __syncthreads();\n"
-      << "    const int t = s_t;\n"
+      << "    const unsigned int t = s_t;\n"
       << "    __syncthreads();\n"
-      << "    if (t >= n_tiles) return;\n"
+      << "    if (t >= (unsigned int)n_tiles) return;\n"
       << "    const BTile tl = tiles[t];\n"
       << "    if ((int)threadIdx.x < tl.count) cs_run(A, tl.prog, tl.first + threadIdx.x);\n"
       << "  }\n}\n";
@@ -266,7 +266,10 @@ cusadi_status batch_device(cusadi_batch b, BatchDev** out) {
     }
   }
   if ((ce = cudaMalloc((void**)&d.d_ticket, 256)) != cudaSuccess) return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
-  if ((ce = cudaMemset(d.d_ticket, 0, 256)) != cudaSuccess) return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
+  // the tables' copies and this memset run on the default stream, which a launch on a
+  // non-blocking stream does not wait for: the host does, once
+  if ((ce = cudaMemset(d.d_ticket, 0, 256)) != cudaSuccess || (ce = cudaStreamSynchronize(nullptr)) != cudaSuccess)
+    return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
   if ((ce = cudaStreamCreateWithFlags(&d.cap, cudaStreamNonBlocking)) != cudaSuccess)
     return bfail(CUSADI_E_CUDA, cudaGetErrorString(ce));
   if (b->n_sat > 0) {

@@ -174,3 +174,21 @@ def test_uneven_batch_at_stated_sizes_against_the_oracle():
     # shallow programs meet the plain tolerance everywhere, the deepest almost nowhere
     assert frac_tau[0] == 1.0 and frac_tau[1] == 1.0, frac_tau
     assert frac_tau[-1] < 0.2, frac_tau
+
+
+def test_first_evaluation_on_a_side_stream_behind_a_busy_default_stream():
+    """The tile table and the tile counter are there before the first launch, whatever
+    stream it goes to and whatever the default stream still has to do."""
+    irs = [programs.random_program(n, seed=100 + j).to_bytes() for j, (n, _) in enumerate(SIZES)]
+    xs, outs, _ = _buffers(irs)
+    plain = [torch.empty_like(o) for o in outs]
+    b = Batch(irs, [N for _, N in SIZES], dtype="f32", segment_ops=2000)
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(100_000_000)           # about 50 ms
+    with torch.cuda.stream(side):
+        b(xs, outs)
+    torch.cuda.synchronize()
+    b(xs, plain, mode="plain")
+    for a, c in zip(outs, plain):
+        assert torch.equal(a, c)
