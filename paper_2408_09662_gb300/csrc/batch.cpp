@@ -319,7 +319,10 @@ cusadi_status launch_scheduler(cusadi_batch b, BatchDev& d, int v, const std::ve
   int nt = (int)b->tiles[v].size();
   if (nt == 0) return CUSADI_OK;
   BArgs t = table(args);
-  void* kargs[] = {&d.d_tiles[v], &nt, &d.d_ticket, &t};
+  // a counter for each tile size: launches of one size leave theirs at zero even when
+  // calls overlap against the rule, since as many CTAs leave as their tickets count
+  unsigned* ticket = d.d_ticket + v;
+  void* kargs[] = {&d.d_tiles[v], &nt, &ticket, &t};
   CUresult r = driver().launchKernel(d.persist[v], (unsigned)d.grid[v], 1, 1, (unsigned)kBlocks[v], 1, 1, 0u,
                                      (CUstream)st, kargs, nullptr);
   return r == CUDA_SUCCESS ? CUSADI_OK : bfail(CUSADI_E_CUDA, "cuLaunchKernel failed: " + std::to_string(r));

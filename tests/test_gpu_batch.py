@@ -192,3 +192,33 @@ def test_first_evaluation_on_a_side_stream_behind_a_busy_default_stream():
     b(xs, plain, mode="plain")
     for a, c in zip(outs, plain):
         assert torch.equal(a, c)
+
+
+def test_overlapping_calls_do_not_spoil_later_ones(batch):
+    """Calls on one batch must not overlap; the results of two that did are undefined, but
+    the next call evaluates every tile again, whatever tile sizes they had."""
+    irs, b = batch
+    xs, outs, _ = _buffers(irs)
+    b(xs, outs, mode="plain")
+    want = [o.clone() for o in outs]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    for trial in range(40):                 # the second starts a little later each time
+        gate = torch.cuda.Event()
+        torch.cuda._sleep(1_000_000)
+        gate.record()
+        for st, block, wait in ((streams[0], 32, 0), (streams[1], 128, 8_000 * trial)):
+            st.wait_event(gate)
+            b.set_block(block)
+            with torch.cuda.stream(st):
+                if wait:
+                    torch.cuda._sleep(wait)
+                b(xs, outs)
+        torch.cuda.synchronize()
+        for block in (32, 128, 32, 128):
+            b.set_block(block)
+            for o in outs:
+                o.fill_(float("nan"))
+            b(xs, outs)
+            torch.cuda.synchronize()
+            for o, w in zip(outs, want):
+                assert torch.equal(o, w), (trial, block)
