@@ -210,6 +210,7 @@ constexpr int64_t kInterpFew = 152 * 32;
 
 // launchers implemented in kernels.cu.  Input rows >= split are read from X2
 // (row - split); returns a cudaError_t value.
+int prepare_interp(int dtype);   // once per device, before its first launch
 int launch_interp(const IOp* ops, const int32_t* begin, int ways, const void* k, int dtype, const void* X,
                   int64_t ldx, const void* X2, int64_t ldx2, int64_t split, void* Y, int64_t ldy,
                   int64_t N, void* W, int64_t ldw, int64_t n_shared, int acc, int reduce,

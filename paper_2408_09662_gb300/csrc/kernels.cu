@@ -228,10 +228,6 @@ int launch(const IOp* ops, const int32_t* begin, int ways, const void* k, const 
   auto kern = interp_kernel<B, S, MIXED>;
   const int groups = ways == 1 && (size_t)n_shared * 128 * sizeof(S) <= 160 * 1024 ? 4 : 1;   // per CTA
   const size_t smem = (size_t)groups * ((size_t)n_shared * 32 * sizeof(S) + (size_t)ways * 64 * sizeof(uint4));
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return (int)e;
-  }
   const long long grid = (N + 32 * groups - 1) / (32 * groups);
   kern<<<(unsigned)grid, 32 * ways * groups, smem, st>>>(reinterpret_cast<const uint4*>(ops), begin, ways, (const S*)k,
                                                 (const B*)X, ldx, (const B*)X2, ldx2, split, (B*)Y,
@@ -282,6 +278,19 @@ __global__ void __launch_bounds__(512) sum_rows_kernel(const T* __restrict__ Y, 
 }
 
 }  // namespace
+
+// The shared-memory limit belongs to the kernel, which all functions and threads share:
+// it is the device's own, set before the first launch and never lowered to one launch's.
+int prepare_interp(int dtype) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return (int)e;
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (dtype == CUSADI_F64) return (int)cudaFuncSetAttribute(interp_kernel<double, double, false>, attr, most);
+  if (dtype == CUSADI_F32) return (int)cudaFuncSetAttribute(interp_kernel<float, float, false>, attr, most);
+  return (int)cudaFuncSetAttribute(interp_kernel<float, double, true>, attr, most);
+}
 
 int launch_interp(const IOp* ops, const int32_t* begin, int ways, const void* k, int dtype, const void* X,
                   int64_t ldx, const void* X2, int64_t ldx2, int64_t split, void* Y, int64_t ldy,

@@ -390,6 +390,7 @@ cusadi_status load_on_device(cusadi_fn fn, DevState& ds, bool adjoint) {
   }
   Direction& d = adjoint ? fn->adj : fn->fwd;
   if (fn->path == CUSADI_PATH_INTERP) {
+    if (int rc = prepare_interp(fn->opt.dtype)) return cuda_fail("cudaFuncSetAttribute", rc);
     for (int v = 0; v < 2; ++v) {
       const InterpProgram& ip = v ? d.ip_few : d.ip;
       void* ops = nullptr;

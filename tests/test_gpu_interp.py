@@ -2,12 +2,15 @@
 every instance has the same bits whichever layout, shared-memory budget, batch
 size or position it is evaluated in, and the results match the oracle within
 the FP64 rule (FP32 rule for FP32)."""
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
 from oracle import Oracle, tolerance
-from paper_2408_09662_gb300 import inputs, programs
+from paper_2408_09662_gb300 import _lib as L, inputs, programs
 from paper_2408_09662_gb300.api import Function
 from paper_2408_09662_gb300.experiments import _spd
 
@@ -74,3 +77,45 @@ def test_adjoint_layouts_agree(dtype):
         fn.adjoint(x[:, :k].contiguous(), b[:, :k].contiguous(), shared_out=g)
         want = many[:144, :k].double().sum(1)
         assert torch.all((g[:144].double() - want).abs() <= tol * many[:144, :k].double().abs().sum(1) + 1e-30)
+
+
+HAMMER = r"""
+#include <cstdint>
+#include <thread>
+typedef int (*eval_t)(void*, const void*, int64_t, void*, int64_t, int64_t, void*, void*);
+extern "C" int hammer(eval_t eval, void** fn, const void* x, void** y, void** ws, void** stream, int64_t n) {
+  int status[2] = {0, 0};
+  std::thread t[2];
+  for (int k = 0; k < 2; ++k)
+    t[k] = std::thread([&, k] {
+      for (int i = 0; i < 20000 && !status[k]; ++i) status[k] = eval(fn[k], x, n, y[k], n, n, ws[k], stream[k]);
+    });
+  for (auto& u : t) u.join();
+  return status[0] ? status[0] : status[1];
+}
+"""
+
+
+def test_two_threads_with_layouts_of_different_size(tmp_path):
+    """Several host threads may evaluate at once: a launch that needs little shared memory
+    does not lower the limit of the interpreter kernel under another thread's launch."""
+    (tmp_path / "hammer.cpp").write_text(HAMMER)
+    so = str(tmp_path / "hammer.so")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-pthread", "-o", so, str(tmp_path / "hammer.cpp")], check=True)
+    ir, make = program("ldlt22")
+    n = 64
+    x = torch.tensor(make(n), device="cuda")
+    fns = [Function(ir.to_bytes(), dtype="f64", path="interp", interp_shared_kb=kb) for kb in (12, 48)]
+    want = fns[0](x)
+    assert torch.equal(fns[1](x), want)
+    ys, ws = [torch.empty_like(want) for _ in fns], [f.workspace(n, False, "cuda") for f in fns]
+    streams = [torch.cuda.Stream() for _ in fns]
+    torch.cuda.synchronize()
+    two = ctypes.c_void_p * 2
+    status = ctypes.CDLL(so).hammer(
+        ctypes.cast(L.lib().cusadi_eval, ctypes.c_void_p), two(*[f.handle for f in fns]), ctypes.c_void_p(x.data_ptr()),
+        two(*[y.data_ptr() for y in ys]), two(*[w.data_ptr() if w is not None else None for w in ws]),
+        two(*[s.cuda_stream for s in streams]), ctypes.c_int64(n))
+    torch.cuda.synchronize()
+    assert status == 0
+    assert all(torch.equal(y, want) for y in ys)
