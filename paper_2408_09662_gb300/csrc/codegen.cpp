@@ -180,8 +180,9 @@ const char* const kSincosF = "static __device__ __noinline__ float2 cs_sincos_f(
 // the halves (|c r - 1| <= 2^-25, or the sum with l: 1 when rounded) and no other.
 // Overflow: a product past the largest finite value (c < 1) stays there, and the
 // residual decides.  An infinite x, whose residual is a NaN otherwise, stays.
-// Bits of x / c for 2^-20 <= c < 2^24.  SRB step FP32, 75 such divisions, N = 4,096: 6.49
-// -> 5.88 us, its adjoint 15.1 -> 13.2, N = 65,536: 9.1 -> 8.4 and 35.6 -> 30.5.
+// Bits of x / c for 2^-20 <= c < 2^24 (powers of two: exact_reciprocal).  SRB step FP32,
+// 75 such divisions, N = 4,096: 6.49 -> 5.88 us, its adjoint 15.1 -> 13.2, N = 65,536: 9.1
+// -> 8.4 and 35.6 -> 30.5.
 const char* const kDivc = R"(static __device__ __forceinline__ float cs_divc_f(float x, float c, float r, bool even) {
   const bool t = fabsf(x) < 1.0f, small = c < 1.0f;
   const float S = t ? 0x1p+64f : 1.0f, p = __fmul_rn(x, r);
@@ -208,10 +209,18 @@ uint64_t recip_of(double b) {
   if (m == 1ull << 52) return ~0ull;
   return (uint64_t)(((unsigned __int128)1 << 116) / m);
 }
+// 1/k of a constant power of two, where it is as exact as the division and one multiply;
+// 0: k is none, or its reciprocal no normal number
+double exact_reciprocal(const Node& b, bool f64) {
+  int e;
+  const double k = f64 ? b.k : (double)(float)b.k;
+  if (b.op != CONST || std::fabs(std::frexp(k, &e)) != 0.5 || std::abs(e - 1) > (f64 ? 1022 : 126)) return 0.0;
+  return 1.0 / k;
+}
 // divisors that the constant form takes: normal, and inside cs_div_far's range
 bool const_divisor(const Node& b) {
   const double m = std::fabs(b.k);
-  return b.op == CONST && m >= 0x1p-509 && m < 0x1p+513;
+  return b.op == CONST && m >= 0x1p-509 && m < 0x1p+513 && exact_reciprocal(b, true) == 0.0;
 }
 
 // the function itself, to be inlined where it is named
@@ -334,6 +343,10 @@ std::string op_expr(Gen& G, const Node& x, bool f, const std::string& A, const s
   std::string e;
   MathFn m = math_name(x.op);
   const char* mn = f ? m.d : m.f;
+  if (x.op == DIV) {
+    const double r = exact_reciprocal(G.g.nodes[x.b], f);
+    if (r != 0.0) return A + " * " + lit(r, f);
+  }
   if (f && own_f64_math(x.op)) {
     const int op = x.op == INV ? (int)DIV : (int)x.op;
     const bool inl = inlined(op, o.inline_math);

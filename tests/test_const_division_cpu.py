@@ -3,6 +3,8 @@ host: the bits of x / c."""
 import re
 import subprocess
 
+import pytest
+
 from paper_2408_09662_gb300 import tracer as T
 from paper_2408_09662_gb300.api import Function
 
@@ -78,3 +80,18 @@ SUBNORMAL = ("for (int i = 0; i < 4000; ++i) { const double h = ((double)(g() % 
 
 def test_subnormal_quotients(tmp_path):
     assert differences(tmp_path, SUBNORMAL + EVERY_EXPONENT.replace("KEEP", "true")) == ""
+
+
+@pytest.mark.parametrize("ways", [0, 2])
+@pytest.mark.parametrize("dtype,least,most", [("f64", -1022, 1022), ("f32", -126, 126)])
+def test_division_by_a_power_of_two_is_a_multiply(dtype, least, most, ways):
+    """Where the reciprocal is a normal number: exact, and free to join an add."""
+    (x,) = T.Graph().symbols(1)
+    k = [2.0, -0.25, 2.0 ** least, 2.0 ** most]
+    src = Function(T.Function([("x", [x])], [("y", [x / c for c in k])]).to_ir(), dtype=dtype, ways=ways, cache_dir=None).source()
+    suffix = "f" if dtype == "f32" else ""
+    for r in ("0x1p-1", "-0x1p+2", f"0x1p{-least:+d}", f"0x1p{-most:+d}"):
+        assert f" * ({r}{suffix});" in src, r
+    assert not re.search(r"= v\w+ / |cs_div\w*\(v", src)
+    beyond = Function(T.Function([("x", [x])], [("y", [x / 2.0 ** (least - 1)])]).to_ir(), dtype=dtype, ways=ways, cache_dir=None)
+    assert " * (0x" not in beyond.source()
