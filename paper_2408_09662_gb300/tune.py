@@ -10,8 +10,9 @@ configurations (concurrently: the compiles release the GIL), times each on the
 caller's own batch (CUDA events on the current stream, L2 flushed before every
 launch, median of `reps`) and keeps the fastest.  The choice is cached on disk
 keyed by the program's content hash, the GPU, the dtype, the batch size (to
-the next power of two) and the caller's fixed options, so a later call loads
-the chosen kernel directly.
+the next power of two), the caller's fixed options and the engine's sources (what
+other code was timed with says nothing about these kernels), so a later call
+loads the chosen kernel directly.
 
 Search, in three rounds:
 1. shape: ways in `ways` (0 = one thread per instance, W = W warps per group
@@ -27,6 +28,7 @@ budget, spill_values, measured no faster on any program and are not searched.)
 """
 from __future__ import annotations
 
+import functools
 import hashlib
 import json
 import os
@@ -37,6 +39,7 @@ from concurrent.futures import ThreadPoolExecutor
 import torch
 
 from .api import DEFAULT_CACHE, Function, _program_bytes
+from .build import _sources
 
 
 def _refinements(best: dict, dtype: str, n_ops: int, n_slots: int, adjoint: bool = False) -> list:
@@ -58,12 +61,22 @@ def _refinements(best: dict, dtype: str, n_ops: int, n_slots: int, adjoint: bool
     return out
 
 
+@functools.lru_cache(maxsize=None)
+def _engine() -> str:
+    """Hash of the library's sources."""
+    h = hashlib.sha256()
+    for path in _sources():
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
 def _key(ir: bytes, dtype: str, N: int, fixed: dict, device, target: str = "eval") -> str:
     props = torch.cuda.get_device_properties(device)
     bucket = 1 << max(0, (int(N) - 1).bit_length())
     h = hashlib.sha256(ir).hexdigest()[:20]
     fx = ",".join(f"{k}={fixed[k]}" for k in sorted(fixed))
-    key = f"{h}|{props.name}|sm_{props.major}{props.minor}|{dtype}|N<={bucket}|{fx}"
+    key = f"{h}|{props.name}|sm_{props.major}{props.minor}|{dtype}|N<={bucket}|{fx}|engine {_engine()}"
     return key if target == "eval" else key + "|" + target
 
 

@@ -62,3 +62,18 @@ def test_cache_file_round_trip(tmp_path):
     assert d["k1"]["options"] == {"ways": 4} and d["k2"]["ms"] == 2.0
     open(path, "w").write("{not json")
     assert tune._load_cache(path) == {}          # a damaged file is ignored, not fatal
+
+
+def test_cache_key_follows_the_engine(monkeypatch):
+    """A choice timed with other sources of the library is not taken for this one's."""
+    import types
+    import torch
+    from paper_2408_09662_gb300 import tune
+    monkeypatch.setattr(torch.cuda, "get_device_properties", lambda device: types.SimpleNamespace(name="GB300", major=10, minor=3))
+    k = tune._key(b"program-a", "f64", 4096, {}, "cuda:0")
+    assert k == tune._key(b"program-a", "f64", 4096, {}, "cuda:0")
+    monkeypatch.setattr(tune, "_sources", lambda: [__file__])
+    tune._engine.cache_clear()
+    other = tune._key(b"program-a", "f64", 4096, {}, "cuda:0")
+    tune._engine.cache_clear()
+    assert other != k
