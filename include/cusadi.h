@@ -94,7 +94,9 @@ typedef struct {
                                  win: time it); 0: one instance per thread (an FP64
                                  program of 64 to 6,000 ops, other launch options at
                                  their defaults, runs as ways = 8 on as few instances as
-                                 the GPU holds at once that way: 4,864 to 19,456)   (0) */
+                                 the GPU holds at once that way: 4,864 to 19,456; an
+                                 instance's results have the same bits at every batch
+                                 size)                                              (0) */
   int32_t own_math;           /* FP32 sin/cos/exp: 0 the library's (out-of-line calls),
                                  1 the engine's own (<= 2 ulp) inlined, 2 the engine's
                                  own as out-of-line functions                      (0) */

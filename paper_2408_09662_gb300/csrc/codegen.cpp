@@ -109,7 +109,10 @@ struct Gen {
   const char* ty(bool f64) const { return f64 ? "double" : "float"; }
   bool buf_f64() const { return o.dtype == CUSADI_F64; }
   bool ws_f64() const { return o.dtype != CUSADI_F32; }
-  bool leaf(int32_t i) const { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; }
+  // no value of its own to compute: inputs, constants, multiplies that joined their readers
+  bool leaf(int32_t i) const {
+    return g.nodes[i].op == INPUT || g.nodes[i].op == CONST || (!g.gone.empty() && g.gone[i]);
+  }
 };
 
 // Whether op is inlined at its uses (else one out-of-line function per op and
@@ -335,10 +338,24 @@ static __device__ __forceinline__ void cs_st4(double* __restrict__ p, bool full,
 }
 )";
 
-// C expression of one op with operand expressions A, B in precision f.
-std::string op_expr(Gen& G, const Node& x, bool f, const std::string& A, const std::string& B,
+// C expression of node i, in precision f, with its operands' expressions (operands()).
+std::string op_expr(Gen& G, int64_t i, bool f, const std::string& A, const std::string& B, const std::string& C,
                     const CodegenOptions& o) {
+  const Node& x = G.g.nodes[i];
   const char* T = G.ty(f);
+  if (!G.g.fused.empty()) {   // contraction decided: nothing is left to the compiler
+    const int32_t m = G.g.fused[i];
+    const std::string rn = f ? "_rn(" : "f_rn(", d = f ? "__d" : "__f";
+    if (m >= 0) {
+      const std::string& F = G.g.nodes[m].op == SQ ? A : B;
+      return std::string(f ? "fma(" : "fmaf(") + (x.op == SUB && x.b == m ? "-" : "") + A + ", " + F + ", " +
+             (x.op == SUB && x.a == m ? "-" : "") + C + ")";
+    }
+    const double r = x.op == DIV ? exact_reciprocal(G.g.nodes[x.b], f) : 0.0;
+    if (r != 0.0) return d + "mul_rn(" + A + ", " + lit(r, f) + ")";
+    if (x.op == MUL || x.op == SQ) return d + "mul_rn(" + A + ", " + (x.op == SQ ? A : B) + ")";
+    if (x.op == ADD || x.op == SUB) return d + (x.op == ADD ? "add_rn(" : "sub_rn(") + A + ", " + B + ")";
+  }
   std::string Z = std::string("(") + T + ")0", One = std::string("(") + T + ")1";
   std::string e;
   MathFn m = math_name(x.op);
@@ -448,7 +465,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   for (int64_t i = 0; i < n; ++i) {
     const Node& x = g.nodes[i];
     if (G.leaf(i)) continue;
-    for (int32_t a : {x.a, x.b})
+    for (int32_t a : operands(g, i))
       if (a >= 0 && !G.leaf(a)) G.last_seg[a] = std::max(G.last_seg[a], G.seg_of[i]);
   }
   // workspace rows for values read in a later segment; a row is free again for
@@ -622,8 +639,8 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
   std::vector<int64_t> waits(n, -1);           // division evaluated with a later one
   std::vector<int64_t> first_use(n, INT64_MAX);
   for (int64_t i = n - 1; i >= 0; --i)
-    for (int32_t a : {g.nodes[i].a, g.nodes[i].b})
-      if (a >= 0) first_use[a] = i;
+    for (int32_t a : operands(g, i))
+      if (a >= 0 && !G.leaf(i)) first_use[a] = i;
   auto short_div = [&](int64_t i) -> int32_t {
     const Node& x = g.nodes[i];
     if (G.leaf(i) || (x.op != DIV && x.op != INV) || !G.node_f64((int32_t)i)) return -1;
@@ -819,6 +836,7 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
       const Node& x = g.nodes[i];
       const bool f = G.node_f64((int32_t)i);
       const char* T = G.ty(f);
+      const std::array<int32_t, 3> reads = operands(g, i);
       if (waits[i] >= 0) continue;   // evaluated with a later division
       const bool two_div = partner[i] >= 0 && short_div(i) >= 0;
       const bool sincos = partner[i] >= 0 && !two_div && g.nodes[partner[i]].op != x.op;
@@ -876,9 +894,10 @@ CodegenResult generate(const Graph& g, const CodegenOptions& o) {
         have_recip[dv] = 1;
       } else {
         for (int l = 0; l < NL; ++l) {
-          std::string A = x.a >= 0 ? operand(x.a, f, l) : "";
-          std::string B = x.b >= 0 ? operand(x.b, f, l) : "";
-          body << "  const " << T << " " << vname(i, l) << " = " << op_expr(G, x, f, A, B, o) << ";\n";
+          std::string e[3];
+          for (int k = 0; k < 3; ++k)
+            if (reads[k] >= 0) e[k] = operand(reads[k], f, l);
+          body << "  const " << T << " " << vname(i, l) << " = " << op_expr(G, i, f, e[0], e[1], e[2], o) << ";\n";
         }
       }
       keep(i);
@@ -1068,8 +1087,7 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
     if (!G.leaf(i)) G.seg_of[i] = seg_of_phase[plan.phase[i]];
   for (int64_t i = 0; i < n; ++i) {
     if (G.leaf(i)) continue;
-    const Node& x = g.nodes[i];
-    for (int32_t a : {x.a, x.b})
+    for (int32_t a : operands(g, i))
       if (a >= 0 && !G.leaf(a)) G.last_seg[a] = std::max(G.last_seg[a], G.seg_of[i]);
   }
   std::vector<int> slot, gslot;
@@ -1155,8 +1173,7 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
     std::vector<int> last_own_phase(n, -1);
     for (int64_t i = 0; i < n; ++i) {
       if (G.leaf(i) || G.seg_of[i] != s) continue;
-      const Node& x = g.nodes[i];
-      for (int32_t a : {x.a, x.b})
+      for (int32_t a : operands(g, i))
         if (a >= 0 && !G.leaf(a) && G.seg_of[a] == s && plan.owner[a] == plan.owner[i])
           last_own_phase[a] = std::max(last_own_phase[a], plan.phase[i]);
     }
@@ -1205,17 +1222,19 @@ CodegenResult generate_coop(const Graph& g, const CodegenOptions& o, const CoopP
       const int nph = nph_seg;
       for (int q = 0; q < nph; ++q) {
         for (int64_t i : work[w][q]) {
-          const Node& x = g.nodes[i];
           const bool f = G.node_f64((int32_t)i);
           const char* T = G.ty(f);
-          std::string A = x.a >= 0 ? operand(x.a, f) : "";
-          std::string B = x.b >= 0 ? operand(x.b, f) : "";
+          const std::array<int32_t, 3> reads = operands(g, i);
+          std::string e[3];
+          for (int k = 0; k < 3; ++k)
+            if (reads[k] >= 0) e[k] = operand(reads[k], f);
+          const std::string value = op_expr(G, i, f, e[0], e[1], e[2], o);
           const bool persists = plan.phase[i] < last_own_phase[i];
           if (persists) {
             decls << "  " << T << " v" << i << ";\n";
-            body << "    v" << i << " = " << op_expr(G, x, f, A, B, o) << ";\n";
+            body << "    v" << i << " = " << value << ";\n";
           } else {
-            body << "    const " << T << " v" << i << " = " << op_expr(G, x, f, A, B, o) << ";\n";
+            body << "    const " << T << " v" << i << " = " << value << ";\n";
           }
           have[i] = 1;
           if (slot[i] >= 0) body << "    cs_x[" << slot[i] << " * 32 + lane] = (" << tsm << ")v" << i << ";\n";

@@ -56,7 +56,9 @@ double barrier_cost(int dtype) {
   return c >= 0 ? c : (dtype == CUSADI_F64 ? 78.0 : 6.0);
 }
 
-bool is_leaf(const Graph& g, int64_t i) { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; }
+bool is_leaf(const Graph& g, int64_t i) {   // no value of its own to compute (Gen::leaf)
+  return g.nodes[i].op == INPUT || g.nodes[i].op == CONST || (!g.gone.empty() && g.gone[i]);
+}
 
 struct Ready {
   double pri;
@@ -175,7 +177,7 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
   for (int64_t i = 0; i < n; ++i) {
     const Node& x = g.nodes[i];
     if (is_leaf(g, i)) { d.skip[i] = 1; continue; }
-    if (x.op != ADD && x.op != SUB) continue;
+    if ((x.op != ADD && x.op != SUB) || !g.fused.empty()) continue;   // else contract() has decided
     for (int32_t m : {x.a, x.b})
       if (fused[i] < 0 && (g.nodes[m].op == MUL || g.nodes[m].op == SQ) && reads[m] == 1 &&
           g.nodes[m].f64 == x.f64 && (dtype == CUSADI_F64 || (dtype == CUSADI_MIXED && x.f64))) {
@@ -188,7 +190,8 @@ CoopPlan plan_coop(const Graph& g, int ways, double comm_cost, int dtype) {
     const Node& x = g.nodes[i];
     const int32_t m = fused[i];
     d.cost[i] = op_cost(x, dtype);
-    const int32_t o[3] = {m < 0 ? x.a : g.nodes[m].a, m < 0 ? x.b : g.nodes[m].b, m < 0 ? -1 : (x.a == m ? x.b : x.a)};
+    std::array<int32_t, 3> o = operands(g, i);
+    if (m >= 0) o = {g.nodes[m].a, g.nodes[m].b, x.a == m ? x.b : x.a};
     for (int k = 0; k < 3; ++k) d.deps[i][k] = o[k] >= 0 && !is_leaf(g, o[k]) ? o[k] : -1;
   }
   d.finish();
@@ -256,14 +259,13 @@ int assign_coop_slots(const Graph& g, const CoopPlan& P, const std::vector<int>&
   // value goes to a workspace row instead (the CTA barrier orders global
   // memory as well).  Reads from a later kernel go through the workspace.
   const int64_t n = (int64_t)g.nodes.size();
-  auto leaf = [&](int64_t i) { return g.nodes[i].op == INPUT || g.nodes[i].op == CONST; };
+  auto leaf = [&](int64_t i) { return is_leaf(g, i); };
   slot.assign(n, -1);
   gslot.assign(n, -1);
   std::vector<int> last_read(n, -1);
   for (int64_t i = 0; i < n; ++i) {
     if (leaf(i)) continue;
-    const Node& x = g.nodes[i];
-    for (int32_t o : {x.a, x.b})
+    for (int32_t o : operands(g, i))
       if (o >= 0 && !leaf(o) && P.owner[o] != P.owner[i] && seg_of_node[o] == seg_of_node[i])
         last_read[o] = std::max(last_read[o], P.phase[i]);
   }

@@ -64,6 +64,10 @@ struct Graph {
   std::vector<int32_t> out;      // node of each stacked output row
   std::vector<uint8_t> out_reduce;  // per output row: summed over instances (adjoint)
   std::vector<uint8_t> in_bcast;    // per stacked input row: broadcast
+  // filled by contract() (else empty): per add or subtract the multiply that it
+  // evaluates with one rounding, -1; per multiply whether every reader does so
+  std::vector<int32_t> fused;
+  std::vector<uint8_t> gone;
   int64_t nnz_in = 0;
 };
 
@@ -72,6 +76,11 @@ Graph build_ssa(const IRFile& f);
 void simplify(Graph& g, int dtype);
 // Reorders nodes to lower the number of simultaneously live values.
 void schedule(Graph& g);
+// Decides which multiplies join the adds and subtracts that read them (g.fused).
+void contract(Graph& g, int dtype);
+// Values that node i reads: with a multiply joined, its factors (the second -1 for a
+// square) and the other operand of the add.
+std::array<int32_t, 3> operands(const Graph& g, int64_t i);
 // Reverse-mode transform: inputs [x (nnz_in rows); y_bar (nnz_out rows)],
 // outputs x_bar (nnz_in rows); broadcast x rows are marked out_reduce.
 Graph adjoint_graph(const Graph& g);

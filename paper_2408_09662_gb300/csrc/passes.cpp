@@ -528,4 +528,44 @@ Graph adjoint_graph(const Graph& fwd) {
   return g;
 }
 
+// A program that runs in one of several kernels by the size of the batch gives every
+// instance the same bits in each: which multiplies round on their own is decided here
+// for all of them, since the compiler's choice changes with the register bound and with
+// what a warp holds.  It is the compiler's rule otherwise: a multiply (no output) whose
+// readers, at most four, are all adds and subtracts joins them; one with a single
+// reader first, one reader joins one.
+void contract(Graph& g, int dtype) {
+  const int64_t n = (int64_t)g.nodes.size();
+  g.fused.assign(n, -1);
+  g.gone.assign(n, 0);
+  std::vector<std::vector<int32_t>> readers(n);
+  for (int64_t i = 0; i < n; ++i)
+    for (int32_t a : {g.nodes[i].a, g.nodes[i].b})
+      if (a >= 0 && readers[a].size() <= 4) readers[a].push_back((int32_t)i);
+  std::vector<uint8_t> output(n, 0);
+  for (int32_t o : g.out) output[o] = 1;
+  for (int pass = 0; pass < 2; ++pass)
+    for (int64_t m = 0; m < n; ++m) {
+      const std::vector<int32_t>& u = readers[m];
+      if ((g.nodes[m].op != MUL && g.nodes[m].op != SQ) || output[m] || g.gone[m]) continue;
+      if (u.empty() || u.size() > (pass == 0 ? 1 : 4)) continue;
+      bool all = true;
+      for (int32_t i : u) {
+        const Node& x = g.nodes[i];
+        all &= (x.op == ADD || x.op == SUB) && x.a != x.b && g.fused[i] < 0 &&
+               (dtype != CUSADI_MIXED || x.f64 == g.nodes[m].f64);
+      }
+      if (!all) continue;
+      for (int32_t i : u) g.fused[i] = (int32_t)m;
+      g.gone[m] = 1;
+    }
+}
+
+std::array<int32_t, 3> operands(const Graph& g, int64_t i) {
+  const Node& x = g.nodes[i];
+  const int32_t m = g.fused.empty() ? -1 : g.fused[i];
+  if (m < 0) return {x.a, x.b, -1};
+  return {g.nodes[m].a, g.nodes[m].b, x.a == m ? x.b : x.a};
+}
+
 }  // namespace cusadi

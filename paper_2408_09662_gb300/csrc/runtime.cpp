@@ -263,6 +263,10 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   co.adjoint = adjoint;
   co.split = adjoint ? fn->ir.nnz_in : -1;
   static const char* tag[] = {"f64", "f32", "mixed"};
+  // FP64 programs with a form of their own for few instances (below)
+  if (fn->opt.dtype == CUSADI_F64 && fn->opt.fmad && co.spill_values == 0 && d.n_ops >= kFewMinOps &&
+      d.n_ops <= kFewOps && (co.segment_ops <= 0 || d.n_ops <= co.segment_ops))
+    contract(d.g, CUSADI_F64);
   co.prefix = std::string(adjoint ? "cs_adj_" : "cs_fwd_") + tag[fn->opt.dtype];
   if (fn->opt.ways > 1) {
     co.prefix = std::string(adjoint ? "cs_coopadj" : "cs_coop") + std::to_string(fn->opt.ways) + "_" +
@@ -290,6 +294,10 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   if (o.dtype == CUSADI_F64 && o.ways == 0 && d.n_ops <= kFewOps && co.inst_per_thread <= 1 &&
       co.sync_every == 0 && co.spill_values == 0 && d.cg.register_cap == 255 && d.cg.segs.size() == 1 &&
       co.maxrregcount == 0) {
+    if (o.fmad && d.g.fused.empty()) {
+      contract(d.g, o.dtype);
+      d.cg = generate(d.g, co);
+    }
     CodegenOptions cm = co;
     cm.prefix = adjoint ? "cs_many_adj_f64" : "cs_many_f64";
     cm.maxrregcount = kManyCap;
@@ -297,6 +305,7 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   } else if (o.dtype != CUSADI_F64 && o.ways == 0 && co.inst_per_thread <= 1 && co.sync_every == 0 &&
              co.spill_values == 0 && co.maxrregcount == 0 && d.cg.register_cap == kManyCap &&
              d.cg.segs.size() == 1) {
+    if (o.fmad) contract(d.g, o.dtype);
     CodegenOptions cm = co;
     cm.prefix = std::string(adjoint ? "cs_many_adj_" : "cs_many_") + tag[o.dtype];
     cm.maxrregcount = kManyCap;

@@ -79,3 +79,23 @@ def test_single_precision_many_at_128_registers(n):
     fn = Function(irb, dtype="f32", fmad=0)
     assert "__launch_bounds__(128) cs_fwd" in fn.source()
     assert torch.equal(fn(x), Function(irb, dtype="f32", fmad=0, maxrregcount=128)(x))
+
+
+@pytest.mark.parametrize("name,dtype", [("cartpole", "f64"), ("srb", "f64"), ("random3k", "f64"), ("random5k", "f32")])
+def test_bits_do_not_depend_on_the_batch_size(name, dtype):
+    """The first n columns of a large batch have the bits of a batch of n: one form for
+    few instances, one for most, one beyond one wave; contraction on (the default)."""
+    ir = {"cartpole": programs.cartpole_rk4, "srb": programs.srb_step, "random3k": lambda: programs.random_program(3000, seed=21),
+          "random5k": lambda: programs.random_program(5000, seed=101)}[name]()
+    fn = Function(ir, dtype=dtype, adjoint=1)
+    N = 65537
+    g = torch.Generator(device="cuda").manual_seed(2)
+    x = (torch.randn((fn.nnz_in, N), generator=g, device="cuda", dtype=torch.float64) * 0.3).to(fn.torch_dtype)
+    b = torch.randn((fn.nnz_out, N), generator=g, device="cuda", dtype=torch.float64).to(fn.torch_dtype)
+    y, xb = fn(x), fn.adjoint(x, b)
+    acc = fn.adjoint(x, b, out=torch.ones_like(x), accumulate=True)
+    for n in (1, 33, FEW, FEW + 1, MANY, MANY + 1, 38912, 38913, 50001):
+        xn, bn = x[:, :n].contiguous(), b[:, :n].contiguous()
+        assert torch.equal(fn(xn), y[:, :n]), n
+        assert torch.equal(fn.adjoint(xn, bn), xb[:, :n]), n
+        assert torch.equal(fn.adjoint(xn, bn, out=torch.ones_like(xn), accumulate=True), acc[:, :n]), n
