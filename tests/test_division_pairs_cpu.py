@@ -48,7 +48,7 @@ def test_a_quotient_that_waits_is_no_argument_before_its_turn():
     load(program(f, 4), schedule=0, pair_calls=64)
 
 
-def random_program(seed, ops):
+def random_program(seed, ops, sines=True):
     """Sums, products, sines and quotients by two inputs and two constants; outputs are
     the values read last."""
     rng = random.Random(seed)
@@ -56,7 +56,7 @@ def random_program(seed, ops):
     v = list(x)
     for _ in range(ops):
         a, b = rng.choice(v[-12:]), rng.choice(v[-12:])
-        v.append(rng.choice([lambda: a + b, lambda: a - b, lambda: a * b, lambda: T.sin(a), lambda: a / x[0],
+        v.append(rng.choice([lambda: a + b, lambda: a - b, lambda: a * b, lambda: T.sin(a) if sines else b - a, lambda: a / x[0],
                              lambda: a / x[1], lambda: a / M, lambda: a / P, lambda: a / P])())
     return T.Function([("x", list(x))], [("y", v[-8:])]).to_ir()
 

@@ -83,3 +83,59 @@ def test_host_build_of_the_fp64_functions(tmp_path):
     bad, worst = subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()
     assert int(bad) == 0
     assert float(worst) <= 0.6
+
+
+# the forms with several results or a divisor used again, against the plain ones
+FORMS = r"""
+int main() {
+  long bad = 0;
+  const double edge[] = {0.0, -0.0, INFINITY, -INFINITY, NAN, 5e-324, -5e-324, 0x1p-1022, 0x1.fffffffffffffp-1023, 0x1p-510,
+                         0x1p-509, 0x1.fffffffffffffp-510, 0x1.fffffffffffffp+512, 0x1p+513, 0x1.fffffffffffffp+1023, 1.0,
+                         -3.0, 0x1.fffffffffffffp+0, 0x1.0000000000001p+0};
+  auto same = [](double a, double b) { return as<u64>(a) == as<u64>(b) || (std::isnan(a) && std::isnan(b)); };
+  auto divide = [&](double a, double c, double b) {
+    const u64 r = cs_recip64(b);
+    double p, q;
+    cs_divr64x2(a, c, b, r, p, q);
+    bad += !same(cs_divr64(a, b, r), a / b) + !same(p, a / b) + !same(q, c / b);
+    u64 u = as<u64>(b) & 0xfffffffffffffull;       // the reciprocal of a constant, as the generator gives it
+    u = u ? (u64)(((unsigned __int128)1 << 116) / (u | 1ull << 52)) : ~0ull;
+    bad += !same(cs_divr64(a, b, u), a / b);
+  };
+  for (off = -1; off <= 1; ++off) {
+    for (double a : edge)
+      for (double c : edge)
+        for (double b : edge) divide(a, c, b);
+    for (int i = 0; i < 300000; ++i) {
+      double a = bits(1, 2046), c = bits(500, 1500), b = bits(400, 1600);
+      if (i % 4 == 0) a = b * (1 + (int)(g() % 5 - 2) * 0x1p-52);
+      if (i % 4 == 1) c = b * (double)(g() % (1 << 20));
+      divide(a, c, b);
+    }
+  }
+  off = 0;
+  auto trig = [&](double x) {
+    double s, c;
+    cs_sincos64(x, s, c);
+    bad += !same(s, cs_sin64(x)) + !same(c, cs_cos64(x));
+  };
+  for (double x : edge) trig(x);
+  for (double x : {0x1p-27, 0x1p+18, 0.5}) for (double y : {x, nextafter(x, 0.0), nextafter(x, 1e9)}) { trig(y); trig(-y); }
+  for (int i = 0; i < 400000; ++i) trig(bits(980, 1042));
+  for (int k = 1; k < 160000; ++k) {               // next to multiples of pi/2
+    const double x = (double)(k * 1.57079632679489661923132169163975144L);
+    trig(x); trig(-x); trig(nextafter(x, 0.0)); trig(nextafter(x, 1e9));
+  }
+  printf("%ld\n", bad);
+}
+"""
+
+
+def test_forms_with_several_results_equal_the_plain_ones(tmp_path):
+    if os.uname().machine != "x86_64":
+        pytest.skip("the extended-precision reference functions are the x87 ones")
+    (tmp_path / "host.cpp").write_text(HOST[:HOST.index("int main()")] + FORMS)
+    exe = str(tmp_path / "host")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-w", "-I", CSRC, "-o", exe, str(tmp_path / "host.cpp")],
+                   check=True)
+    assert int(subprocess.run([exe], check=True, capture_output=True, text=True).stdout) == 0
