@@ -415,7 +415,7 @@ size_t cusadi_batch_workspace_bytes(cusadi_batch b);
  * device loads the modules and uploads the tile table (allocates; not
  * capturable); with satellites, a persistent call on other buffers than the last
  * captures the graph again, since its launches carry the addresses.  Other
- * calls only launch.  The tile counter belongs to the batch (one per device), so
+ * calls only launch.  The tile counters belong to the batch (one per device and tile size), so
  * calls on one batch must not overlap on the GPU: issue them on one stream, or
  * order them with events. */
 cusadi_status cusadi_batch_eval(cusadi_batch b, const void* const* in, const int64_t* ld_in,

@@ -125,8 +125,8 @@ bool inlined(int op, int inline_math) {
 
 // FP64 functions that run on the integer pipe (math64.cuh), where the
 // straight-line kernels leave it idle; an FP64 instruction occupies its unit 64
-// clocks per warp.  Weights in FMAs, library -> ours (see math64.cuh): exp 15,
-// sin/cos 18, div 7.7, sqrt 8.2 -> 1.6 to 4.
+// clocks per warp.  Weights in FMAs, library -> ours, from long chains of one op:
+// exp 15 -> 1.2, sin/cos 18 -> 4.4, div 7.7 -> 1.9, sqrt 8.2 -> 1.9.
 bool own_f64_math(int op) {
   return op == EXP || op == SIN || op == COS || op == DIV || op == INV || op == SQRT;
 }
