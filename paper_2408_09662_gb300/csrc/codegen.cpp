@@ -343,23 +343,16 @@ std::string op_expr(Gen& G, int64_t i, bool f, const std::string& A, const std::
                     const CodegenOptions& o) {
   const Node& x = G.g.nodes[i];
   const char* T = G.ty(f);
-  if (!G.g.fused.empty()) {   // contraction decided: nothing is left to the compiler
-    const int32_t m = G.g.fused[i];
-    const std::string rn = f ? "_rn(" : "f_rn(", d = f ? "__d" : "__f";
-    if (m >= 0) {
-      const std::string& F = G.g.nodes[m].op == SQ ? A : B;
-      return std::string(f ? "fma(" : "fmaf(") + (x.op == SUB && x.b == m ? "-" : "") + A + ", " + F + ", " +
-             (x.op == SUB && x.a == m ? "-" : "") + C + ")";
-    }
-    const double r = x.op == DIV ? exact_reciprocal(G.g.nodes[x.b], f) : 0.0;
-    if (r != 0.0) return d + "mul_rn(" + A + ", " + lit(r, f) + ")";
-    if (x.op == MUL || x.op == SQ) return d + "mul_rn(" + A + ", " + (x.op == SQ ? A : B) + ")";
-    if (x.op == ADD || x.op == SUB) return d + (x.op == ADD ? "add_rn(" : "sub_rn(") + A + ", " + B + ")";
+  const int32_t m = G.g.fused.empty() ? -1 : G.g.fused[i];
+  if (m >= 0) {   // contract() joined a multiply: the compiler contracts nothing itself
+    const std::string& F = G.g.nodes[m].op == SQ ? A : B;
+    return std::string(f ? "fma(" : "fmaf(") + (x.op == SUB && x.b == m ? "-" : "") + A + ", " + F + ", " +
+           (x.op == SUB && x.a == m ? "-" : "") + C + ")";
   }
   std::string Z = std::string("(") + T + ")0", One = std::string("(") + T + ")1";
   std::string e;
-  MathFn m = math_name(x.op);
-  const char* mn = f ? m.d : m.f;
+  const MathFn fn = math_name(x.op);
+  const char* mn = f ? fn.d : fn.f;
   if (x.op == DIV) {
     const double r = exact_reciprocal(G.g.nodes[x.b], f);
     if (r != 0.0) return A + " * " + lit(r, f);

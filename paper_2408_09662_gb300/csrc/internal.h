@@ -76,7 +76,8 @@ Graph build_ssa(const IRFile& f);
 void simplify(Graph& g, int dtype);
 // Reorders nodes to lower the number of simultaneously live values.
 void schedule(Graph& g);
-// Decides which multiplies join the adds and subtracts that read them (g.fused).
+// Decides which multiplies join the adds and subtracts that read them (g.fused); the
+// kernels are then compiled with contraction off.
 void contract(Graph& g, int dtype);
 // Values that node i reads: with a multiply joined, its factors (the second -1 for a
 // square) and the other operand of the add.

@@ -530,10 +530,16 @@ Graph adjoint_graph(const Graph& fwd) {
 
 // A program that runs in one of several kernels by the size of the batch gives every
 // instance the same bits in each: which multiplies round on their own is decided here
-// for all of them, since the compiler's choice changes with the register bound and with
-// what a warp holds.  It is the compiler's rule otherwise: a multiply (no output) whose
-// readers, at most four, are all adds and subtracts joins them; one with a single
-// reader first, one reader joins one.
+// for all of them (they are compiled with contraction off), since the compiler's choice
+// changes with the register bound and with what a warp holds.  A multiply (no output)
+// joins its only reader, an add or subtract; in FP64, where an instruction holds its unit
+// for 64 clocks, also two to four readers that are all adds and subtracts.  Against the
+// compiler's contraction, us: random 3,000 ops N = 65,536 328 -> 326, 5,500 ops 654 ->
+// 645, LDL^T n = 22 361 -> 364, cart-pole 56.6 -> 55.4, SRB adjoint 343 -> 341 (350 with
+// single readers only); FP32 random 20,000 ops 338 -> 341, N = 16,384 254 -> 255 (264 with
+// up to four readers).  Rounded intrinsics (__dmul_rn) in place of the compiler's switch
+// cost random programs 4 %.  The library's functions have the same bits without
+// contraction, FP64 pow excepted (a few results in 10^6 an ulp elsewhere, as accurate).
 void contract(Graph& g, int dtype) {
   const int64_t n = (int64_t)g.nodes.size();
   g.fused.assign(n, -1);
@@ -544,7 +550,7 @@ void contract(Graph& g, int dtype) {
       if (a >= 0 && readers[a].size() <= 4) readers[a].push_back((int32_t)i);
   std::vector<uint8_t> output(n, 0);
   for (int32_t o : g.out) output[o] = 1;
-  for (int pass = 0; pass < 2; ++pass)
+  for (int pass = 0; pass < (dtype == CUSADI_F64 ? 2 : 1); ++pass)
     for (int64_t m = 0; m < n; ++m) {
       const std::vector<int32_t>& u = readers[m];
       if ((g.nodes[m].op != MUL && g.nodes[m].op != SQ) || output[m] || g.gone[m]) continue;

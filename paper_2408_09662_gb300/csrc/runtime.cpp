@@ -322,7 +322,9 @@ cusadi_status compile_direction(cusadi_fn fn, Direction& d, bool adjoint) {
   const size_t ns = jobs.size();
   std::vector<std::string> logs(ns);
   std::vector<uint8_t> ok(ns, 0);
-  auto opts = nvrtc_options(fn->opt);
+  cusadi_options compiler = fn->opt;
+  if (!d.g.fused.empty()) compiler.fmad = 0;   // contract() has decided
+  auto opts = nvrtc_options(compiler);
   int nt = fn->opt.compile_threads > 0 ? fn->opt.compile_threads
                                        : (int)std::max(1u, std::thread::hardware_concurrency());
   nt = (int)std::min<size_t>((size_t)nt, ns);

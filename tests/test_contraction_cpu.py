@@ -1,8 +1,7 @@
 """Which multiplies round on their own in the generated kernels.  A program with
 kernels for few, for most and for many instances has it decided before any of them
-is written, so that every instance has the same bits whatever the batch's size:
-the statements of one value agree between the forms, and nothing is left to the
-compiler."""
+is written (and the compiler's contraction off), so that every instance has the same
+bits whatever the batch's size: the statements of one value agree between the forms."""
 import re
 
 import pytest
@@ -31,10 +30,9 @@ def test_forms_of_one_program_round_the_same_values(make):
     eight = Function(ir, dtype="f64", adjoint=1, ways=8, cache_dir=None)
     for adjoint in (False, True):
         a, b = values(one, adjoint), values(eight, adjoint)
-        plain = {v: e for v, e in a.items() if re.search(r"_rn\(|fma\(", e)}
-        assert len(plain) > 100
+        plain = {v: e for v, e in a.items() if re.search(r" [-+*] |fma\(", e)}
+        assert len(plain) > 100 and sum("fma(" in e for e in plain.values()) > 30
         assert {v: b[v] for v in plain} == plain
-        assert not [e for e in list(a.values()) + list(b.values()) if re.search(r"v\d+ [-+*/] |[-+*/] v\d+", e)]
 
 
 def test_multiplies_join_adds_where_every_reader_is_one():
@@ -48,7 +46,7 @@ def test_multiplies_join_adds_where_every_reader_is_one():
     fn = Function(T.Function([("x", x)], [("y", y)]).to_ir(), dtype="f64", cache_dir=None, schedule=0)
     found = list(values(fn).values())
     assert sum(e.startswith("fma(") for e in found) == 3
-    assert sum(e.startswith("__dmul_rn(") for e in found) == 3
-    assert sum(re.match(r"__d(add|sub)_rn\(", e) is not None for e in found) == 2
+    assert sum(" * " in e for e in found) == 3
+    assert sum(re.match(r"v\d+ [-+] v\d+$", e) is not None for e in found) == 2
     off = Function(T.Function([("x", x)], [("y", y)]).to_ir(), dtype="f64", fmad=0, cache_dir=None, schedule=0)
     assert "fma(" not in off.source()
