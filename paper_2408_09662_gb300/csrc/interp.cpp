@@ -331,6 +331,19 @@ bool pack_interp(const Graph& g, InterpProgram& many, InterpProgram& few, std::s
   };
   const int narrow = n_ops < 200 ? 1 : (dtype == CUSADI_F32 && n_ops > 1000 ? 8 : 4);
   if (!choose(many, narrow, true) || !choose(few, n_ops < 200 ? 1 : (n_ops > 1000 ? 16 : 8), false)) return false;
+  // Ops that need one another in a chain leave warps idle, which hold the places of
+  // further groups: half the warps where the program takes as long with them (35 FP32
+  // quotients in a row, N = 65,536, 4 warps 144 us, one 78; FP64 162 and 91; four such
+  // rows side by side FP32, 8 warps 421 us, 4 warps 254).
+  double work = 0;
+  for (int64_t i = 0; i < P.n; ++i)
+    if (!P.d.skip[i]) work += P.d.cost[i];
+  while (many.ways > 1 && work < 0.6 * many.ways * many.estimate) {
+    InterpProgram p;
+    if (!choose(p, many.ways / 2, true)) return false;
+    if (p.ways != many.ways / 2 || p.estimate > 1.05 * many.estimate) break;
+    many = std::move(p);
+  }
   // workspace rows of the groups in flight: past 256 MB they come from HBM at every
   // use, and one wide group per SM is faster (LDL^T with 100 unknowns, N = 8,192:
   // 124 ms with four narrow groups per SM)

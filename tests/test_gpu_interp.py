@@ -119,3 +119,36 @@ def test_two_threads_with_layouts_of_different_size(tmp_path):
     torch.cuda.synchronize()
     assert status == 0
     assert all(torch.equal(y, want) for y in ys)
+
+
+@pytest.mark.parametrize("rows", [1, 2, 4])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_chains_of_ops_leave_no_places_idle(dtype, rows):
+    """Quotients that need one another, one to four rows of them side by side: the same
+    bits at every batch size, and a batch that fits the GPU with one warp to each row
+    takes about as long as a small one."""
+    from paper_2408_09662_gb300 import tracer as T
+    x = T.Graph().symbols(2 * rows)
+    v = list(x[:rows])
+    for _ in range(100):
+        v = [x[rows + j] / (v[j] + 2.0) + 0.1 for j in range(rows)]
+    fn = Function(T.Function([("x", x)], [("y", v)]).to_ir(), dtype=dtype, path="interp")
+    g = torch.Generator(device="cuda").manual_seed(1)
+    X = torch.rand((2 * rows, 65536 // rows), generator=g, device="cuda", dtype=torch.float64).to(fn.torch_dtype) + 0.5
+    y = fn(X)
+    for n in (1, 33, FEW, FEW + 1, 9000):
+        assert torch.equal(fn(X[:, :n].contiguous()), y[:, :n]), n
+
+    def ms(x):
+        times = []
+        for _ in range(9):
+            s, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            s.record()
+            for _ in range(5):
+                fn(x, out=out[:, :x.shape[1]])
+            e.record()
+            e.synchronize()
+            times.append(s.elapsed_time(e))
+        return sorted(times)[4]
+    out = torch.empty_like(y)
+    assert ms(X) < 1.6 * ms(X[:, :4000].contiguous())
